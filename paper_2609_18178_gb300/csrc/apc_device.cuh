@@ -195,6 +195,50 @@ __device__ __forceinline__ uint64_t digest_term_u16(uint32_t gidx, uint32_t bits
   return z ^ (z >> 31);
 }
 
+// The same term in a keyed form, for runs of 16-bit words whose key offsets
+// differ by multiples of four: the key's two contributions to a term are
+//   m4 = 4 * hi + 1   and   t = (hi ^ top) * 0x1CE4E5B9,
+// the high half's part of the first multiply.  As top < 4 flips only the two
+// low bits of hi, (hi + 4q) ^ top = (hi ^ top) + 4q, so one Key16 per residue
+// mod 4 serves a whole run: offset OFF (a multiple of 4) adds 4 * OFF to m4
+// and OFF * 0x1CE4E5B9 to t, one plain add each, in place of hi, m4, the xor
+// with top and a multiply-add per term.
+struct Key16 {
+  uint32_t m4, t;
+};
+
+// Key16 of the index gidx; top as for digest_term_u16.
+__device__ __forceinline__ Key16 key16(uint32_t gidx, uint32_t one, uint32_t top) {
+  uint32_t hi, m4;
+  asm("mad.lo.u32 %0, %2, %4, %3;\n\t"
+      "mad.lo.u32 %1, %0, 4, %2;"
+      : "=r"(hi), "=r"(m4)
+      : "r"(one), "r"(gidx), "n"(0x9E3779B9u));
+  return Key16{m4, (hi ^ top) * 0x1CE4E5B9u};
+}
+
+// Term of half HALF (0 low, 1 high) of the packed words `pair`.  The half is
+// taken and the increment added by one two-way dot product (dp2a with a unit
+// vector), in place of a mask or shift and an add (4,234 to 4,065 us over
+// 1.81 G elements of bf16 state).
+template <uint32_t OFF, int HALF>
+__device__ __forceinline__ uint64_t digest_term_u16(const Key16 &k, uint32_t pair) {
+  static_assert(OFF % 4 == 0, "a Key16 serves offsets of its own residue mod 4");
+  const uint32_t lo = __dp2a_lo(pair, HALF ? 0x0100u : 0x0001u, 0x7F4A7C15u);
+  const uint32_t l1 = lo ^ (k.m4 + 4u * OFF);
+  uint64_t z;
+  asm("{\n\t.reg .u32 rl, rh, u;\n\t"
+      "mad.lo.u32 u, %1, %3, %4;\n\t"
+      "mul.wide.u32 %0, %1, %2;\n\t"
+      "mov.b64 {rl, rh}, %0;\n\t"
+      "add.u32 rh, rh, u;\n\t"
+      "mov.b64 %0, {rl, rh};\n\t}"
+      : "=l"(z)
+      : "r"(l1), "n"(0x1CE4E5B9u), "n"(0xBF58476Du), "r"(k.t + OFF * 0x1CE4E5B9u));
+  z = MulWide::template mul<0x133111EBu, 0x94D049BBu>(z ^ (z >> 27));
+  return z ^ (z >> 31);
+}
+
 __device__ __forceinline__ bool top_bits_shared(uint32_t B, uint32_t R) { return ((B ^ (B + R)) >> 30) == 0; }
 
 // acc += z (mod 2^64), with the high half's carry-add on the FMA pipe.  Used

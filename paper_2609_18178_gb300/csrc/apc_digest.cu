@@ -3,30 +3,37 @@
 // splitmix64 term per element, so the pass is bound by integer issue, not by
 // HBM.
 //
-// Work split: each buffer's 16-byte aligned body is cut into tiles of
-// kDigestTile elements, and each CTA of a persistent grid takes one
-// contiguous run of the launch's tile space (the runs differ by at most one
-// tile).  Inside its run a CTA finds the buffer of its first tile once, then
-// moves to the next buffer only when it crosses one, carrying the element
-// offset and key forward by a tile per step; this costs measurably fewer
-// integer instructions per tile than striding over the tile space with a
-// grid-wide step, which looks the buffer up and rebuilds the offsets for
-// every tile.
+// Work split: each buffer's 16-byte aligned body is cut into warp tiles of
+// 256 * U elements (U = 4, or 2 for little work: kDigestLong, kDigestShort),
+// and each CTA of a persistent grid takes one contiguous run of the launch's
+// fp32 tiles and one of its bf16 tiles (the CTAs' runs differ by at most one
+// tile).  The kWarps warps of a CTA walk a run interleaved, warp w taking its
+// tiles w, w + kWarps, ..., each on its own: a warp finds a buffer by a
+// binary search when its walk leaves the one before, and inside one only steps
+// a pointer and the key.  The CTA as a whole sweeps one region of memory, and
+// no step waits for another warp.
 //
-// Loads: a thread's part of a tile is kDigestUnroll vectors of 8 words.  All
-// tiles of a buffer but its last are full; they run without per-vector bounds
-// checks, and each thread keeps its next full tile in flight with cp.async
-// into shared-memory slots that only it reads (two stages, no barrier), then
-// folds the current one from there.  A buffer's last tile is loaded straight
-// into registers with per-vector checks, and its scalar head and tail go to
-// the CTA that owns its first tile.  (A CTA-wide bulk-copy pipeline like the
-// commit kernel's measured slower here: its per-tile synchronisation costs
-// issue slots, the one resource this pass is short of.)
+// Why warp tiles: a table of many small buffers is bound by the latency of
+// each buffer's first and last tile, and with tiles of a whole CTA (16,384
+// elements) all its warps paid that latency at once, most of them idle in a
+// partly filled tile.  1,100 tensors of 136 to 20,557 elements (4,400 buffers,
+// 63 MB) took 330 us of kernel time that way and take 56 us by warps.
+//
+// Loads: a thread's part of a tile is U vectors of 8 words.  The tiles are
+// full: they run without per-vector bounds checks, and each thread keeps its
+// next tile in flight with cp.async into shared-memory slots that only it
+// reads (two stages, no barrier), then folds the current one from there.
+// What a buffer holds beyond its full tiles (less than a tile, and the scalar
+// head and tail) is loaded straight into registers by one warp, before the
+// walks: entry e by warp e / grid of CTA e mod grid.  (A CTA-wide bulk-copy
+// pipeline like the commit kernel's measured slower here: its per-tile
+// synchronisation costs issue slots, the one resource this pass is short of.)
 //
 // A thread keeps one running 64-bit sum for the slot of the buffer it is in;
-// all threads of a CTA visit the same tiles, so slot changes are CTA-uniform
-// and the running sum is flushed (warp shuffle reduce, then a shared-memory
-// atomic) only when the CTA moves to a buffer of another slot and at exit.
+// all lanes of a warp visit the same tiles, so slot changes are warp-uniform
+// and the running sum is flushed (shuffle reduce, then a shared-memory
+// atomic) only when the warp moves to a buffer of another slot and at exit.
+// The host orders a launch's buffers by type and slot, so that is rare.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -38,6 +45,23 @@
 namespace apc {
 namespace {
 
+// A lane's words of a tile come in 16-byte groups, group j of all lanes being
+// 512 consecutive bytes: kGroups32 groups of 4 fp32 words, kGroups16 of 8
+// bf16 words.  (With 32 consecutive bytes per lane instead, each 16-byte copy
+// takes half of a 32-byte sector and the other half is fetched again: 3-4%
+// slower.)  U is the launch's vectors of 8 words per lane per tile.
+constexpr uint32_t kSpan16 = 32 * 8, kSpan32 = 32 * 4;  // elements from a lane's group to its next
+constexpr int kWarps = kThreads / 32;
+
+template <int U>
+struct Shape {
+  static constexpr int kGroups16 = U, kGroups32 = 2 * U;
+  static constexpr uint64_t kTile = digest_tile(U);
+  // The keys of a thread's terms in a tile lie in [G0, G0 + span - 1]; with
+  // the increment's carry their high words lie in [B, B + span].
+  static constexpr uint32_t kKeySpan32 = (kGroups32 - 1) * kSpan32 + 4, kKeySpan16 = (kGroups16 - 1) * kSpan16 + 8;
+};
+
 // One digest term of this pass.  The pass is bound by the integer ALU, not
 // by issue, and runs faster with the compiler's own 64-bit multiply.
 template <uint32_t K>
@@ -47,102 +71,138 @@ __device__ __forceinline__ uint64_t term(uint32_t gidx, uint32_t bits, uint32_t 
 
 // The same with SHARED: the caller has checked that all of a thread's terms
 // in the tile share the top two bits of the incremented key high word
-// (top_bits_shared over the keys G0 .. G0 + (kDigestUnroll - 1) * kThreads *
-// kVec + 7) and passes them as `top`, so no term computes hi >> 30 itself.
+// (top_bits_shared over the keys of its groups) and passes them as `top`, so
+// no term computes hi >> 30 itself.
 template <uint32_t K, bool SHARED>
 __device__ __forceinline__ uint64_t vterm(uint32_t gidx, uint32_t bits, uint32_t one, uint32_t top) {
   if constexpr (SHARED) return digest_term<K, MulCompiler>(gidx, bits, one, top);
   else return digest_term<K, MulCompiler>(gidx, bits, one);
 }
 
-// A thread's terms of one fp32 tile (kDigestUnroll vectors of 8 words).
-template <bool SHARED>
-__device__ __forceinline__ void fold32(const uint4 (&x)[kDigestUnroll][2], const bool (&ok)[kDigestUnroll], uint32_t G0,
+// A thread's terms of one fp32 tile.
+template <bool SHARED, int G>
+__device__ __forceinline__ void fold32(const uint4 (&x)[G], const bool (&ok)[G], uint32_t G0,
                                        uint32_t one, uint32_t top, uint64_t &t0, uint64_t &t1) {
 #pragma unroll
-  for (int u = 0; u < kDigestUnroll; ++u) {
-    if (!ok[u]) continue;
-    const uint32_t G = G0 + (uint32_t)(u * kThreads * kVec);
-    t0 += vterm<0, SHARED>(G, x[u][0].x, one, top) + vterm<1, SHARED>(G, x[u][0].y, one, top);
-    t1 += vterm<2, SHARED>(G, x[u][0].z, one, top) + vterm<3, SHARED>(G, x[u][0].w, one, top);
-    t0 += vterm<4, SHARED>(G, x[u][1].x, one, top) + vterm<5, SHARED>(G, x[u][1].y, one, top);
-    t1 += vterm<6, SHARED>(G, x[u][1].z, one, top) + vterm<7, SHARED>(G, x[u][1].w, one, top);
+  for (int j = 0; j < G; ++j) {
+    if (!ok[j]) continue;
+    const uint32_t g = G0 + j * kSpan32;
+    t0 += vterm<0, SHARED>(g, x[j].x, one, top) + vterm<1, SHARED>(g, x[j].y, one, top);
+    t1 += vterm<2, SHARED>(g, x[j].z, one, top) + vterm<3, SHARED>(g, x[j].w, one, top);
   }
 }
 
-// A bf16 word's term: with the shared top bits, the 16-bit form of
-// digest_term_u16 (its increment and first xor-shift take two ALU
-// instructions instead of four).
-template <uint32_t K, bool SHARED>
-__device__ __forceinline__ uint64_t hterm(uint32_t gidx, uint32_t bits, uint32_t one, uint32_t top) {
-  if constexpr (SHARED) return digest_term_u16<K, MulCompiler>(gidx, bits, one, top);
-  else return digest_term<K, MulCompiler>(gidx, bits, one);
-}
-
-// A thread's terms of one bf16 tile (kDigestUnroll vectors of 8 words).
-template <bool SHARED>
-__device__ __forceinline__ void fold16(const uint4 (&x)[kDigestUnroll], const bool (&ok)[kDigestUnroll], uint32_t G0,
-                                       uint32_t one, uint32_t top, uint64_t &t0, uint64_t &t1) {
-#pragma unroll
-  for (int u = 0; u < kDigestUnroll; ++u) {
-    if (!ok[u]) continue;
-    const uint32_t G = G0 + (uint32_t)(u * kThreads * kVec);
-    t0 += hterm<0, SHARED>(G, x[u].x & 0xFFFFu, one, top) + hterm<1, SHARED>(G, x[u].x >> 16, one, top);
-    t1 += hterm<2, SHARED>(G, x[u].y & 0xFFFFu, one, top) + hterm<3, SHARED>(G, x[u].y >> 16, one, top);
-    t0 += hterm<4, SHARED>(G, x[u].z & 0xFFFFu, one, top) + hterm<5, SHARED>(G, x[u].z >> 16, one, top);
-    t1 += hterm<6, SHARED>(G, x[u].w & 0xFFFFu, one, top) + hterm<7, SHARED>(G, x[u].w >> 16, one, top);
+// Group J of a bf16 tile's G groups and those after it, keyed.
+template <int J, int G>
+__device__ __forceinline__ void fold16_keyed(const uint4 (&x)[G], const bool (&ok)[G], const Key16 (&k)[4],
+                                             uint64_t &t0, uint64_t &t1) {
+  constexpr uint32_t off = J * kSpan16;
+  if (ok[J]) {
+    t0 += digest_term_u16<off, 0>(k[0], x[J].x) + digest_term_u16<off, 1>(k[1], x[J].x);
+    t1 += digest_term_u16<off, 0>(k[2], x[J].y) + digest_term_u16<off, 1>(k[3], x[J].y);
+    t0 += digest_term_u16<off + 4, 0>(k[0], x[J].z) + digest_term_u16<off + 4, 1>(k[1], x[J].z);
+    t1 += digest_term_u16<off + 4, 0>(k[2], x[J].w) + digest_term_u16<off + 4, 1>(k[3], x[J].w);
   }
+  if constexpr (J + 1 < G) fold16_keyed<J + 1>(x, ok, k, t0, t1);
 }
 
-// The keys of a thread's terms in a tile lie in [G0, G0 + kTileKeySpan - 1];
-// with the increment's carry their high words lie in [B, B + kTileKeySpan].
-constexpr uint32_t kTileKeySpan = (kDigestUnroll - 1) * kThreads * kVec + kVec;
-
-// One tile of a thread's words: kDigestUnroll vectors of 8, the first at q
-// (element `base` of the buffer), the others kThreads vectors apart.  Only
-// the vectors with ok[u] are loaded and folded.
-__device__ __forceinline__ void tile32(const uint4 *q, const bool (&ok)[kDigestUnroll], uint32_t G0, uint32_t one,
-                                       uint64_t &t0, uint64_t &t1) {
-  uint4 x[kDigestUnroll][2];
+// A thread's terms of one bf16 tile: with SHARED, in the keyed 16-bit form
+// (four keys a tile; 1.81 G elements of bf16 state verified in 4,050 us with
+// the key's part formed for every term, 3,913 with the keyed form's adds on
+// the multiply-add pipe and 3,790 with them left to the compiler).
+template <bool SHARED, int G>
+__device__ __forceinline__ void fold16(const uint4 (&x)[G], const bool (&ok)[G], uint32_t G0,
+                                       uint32_t one, uint32_t top, uint64_t &t0, uint64_t &t1) {
+  if constexpr (SHARED) {
+    const Key16 k[4] = {key16(G0, one, top), key16(G0 + 1, one, top), key16(G0 + 2, one, top), key16(G0 + 3, one, top)};
+    fold16_keyed<0>(x, ok, k, t0, t1);
+  } else {
 #pragma unroll
-  for (int u = 0; u < kDigestUnroll; ++u) {
-    if (ok[u]) {
-      x[u][0] = __ldcs(q + 2 * u * kThreads);
-      x[u][1] = __ldcs(q + 2 * u * kThreads + 1);
+    for (int u = 0; u < G; ++u) {
+      if (!ok[u]) continue;
+      const uint32_t g = G0 + u * kSpan16;
+      t0 += term<0>(g, x[u].x & 0xFFFFu, one) + term<1>(g, x[u].x >> 16, one);
+      t1 += term<2>(g, x[u].y & 0xFFFFu, one) + term<3>(g, x[u].y >> 16, one);
+      t0 += term<4>(g, x[u].z & 0xFFFFu, one) + term<5>(g, x[u].z >> 16, one);
+      t1 += term<6>(g, x[u].w & 0xFFFFu, one) + term<7>(g, x[u].w >> 16, one);
     }
   }
+}
+
+// A thread's terms of the groups with ok[j] of one tile, straight from memory
+// (q: the lane's first group).
+template <int G>
+__device__ __forceinline__ void tile32(const uint4 *q, const bool (&ok)[G], uint32_t G0, uint32_t one, uint64_t &t0,
+                                       uint64_t &t1) {
+  uint4 x[G];
+#pragma unroll
+  for (int j = 0; j < G; ++j)
+    if (ok[j]) x[j] = __ldcs(q + j * 32);
   const uint32_t B = G0 + 0x9E3779B9u;
-  if (top_bits_shared(B, kTileKeySpan)) fold32<true>(x, ok, G0, one, B >> 30, t0, t1);
+  if (top_bits_shared(B, Shape<G / 2>::kKeySpan32)) fold32<true>(x, ok, G0, one, B >> 30, t0, t1);
   else fold32<false>(x, ok, G0, one, 0, t0, t1);
 }
 
-__device__ __forceinline__ void tile16(const uint4 *q, const bool (&ok)[kDigestUnroll], uint32_t G0, uint32_t one,
-                                       uint64_t &t0, uint64_t &t1) {
-  uint4 x[kDigestUnroll];
+template <int G>
+__device__ __forceinline__ void tile16(const uint4 *q, const bool (&ok)[G], uint32_t G0, uint32_t one, uint64_t &t0,
+                                       uint64_t &t1) {
+  uint4 x[G];
 #pragma unroll
-  for (int u = 0; u < kDigestUnroll; ++u) {
-    if (ok[u]) x[u] = __ldcs(q + u * kThreads);
-  }
+  for (int u = 0; u < G; ++u)
+    if (ok[u]) x[u] = __ldcs(q + u * 32);
   const uint32_t B = G0 + 0x9E3779B9u;
-  if (top_bits_shared(B, kTileKeySpan)) fold16<true>(x, ok, G0, one, B >> 30, t0, t1);
+  if (top_bits_shared(B, Shape<G>::kKeySpan16)) fold16<true>(x, ok, G0, one, B >> 30, t0, t1);
   else fold16<false>(x, ok, G0, one, 0, t0, t1);
 }
 
-// Which of a thread's vectors in an entry's last tile lie in its body.
-__device__ __forceinline__ void last_tile_ok(uint64_t base, uint64_t vec_end, bool (&ok)[kDigestUnroll]) {
+__device__ __forceinline__ uint32_t word_at(const DigestEntry &E, uint64_t i) {
+  return E.dtype == 0 ? reinterpret_cast<const uint32_t *>(E.data)[i]
+                      : (uint32_t) reinterpret_cast<const uint16_t *>(E.data)[i];
+}
+
+// Which of a lane's groups lie in the first `count` groups of a tile.
+template <int G>
+__device__ __forceinline__ void groups_ok(uint32_t lane, uint32_t count, bool (&ok)[G]) {
 #pragma unroll
-  for (int u = 0; u < kDigestUnroll; ++u) ok[u] = base + (uint64_t)(u * kThreads) * kVec < vec_end;
+  for (int j = 0; j < G; ++j) ok[j] = j * 32 + lane < count;
+}
+
+// What an entry holds beyond its full tiles, done by one warp: the body's
+// last vectors (fewer than a tile), the scalar head (lanes 0-6) and the scalar
+// tail (lanes 8-14).
+template <int U>
+__device__ __forceinline__ uint64_t remainder(const DigestEntry &E, uint32_t lane, uint32_t one) {
+  const uint64_t body = (E.n - E.head) & ~(uint64_t)(kVec - 1);
+  const uint64_t begin = E.head + body / Shape<U>::kTile * Shape<U>::kTile;
+  const uint32_t rest = (uint32_t)(body % Shape<U>::kTile), G0 = E.key_base + (uint32_t)begin;
+  uint64_t t0 = 0, t1 = 0;
+  if (E.dtype == 0) {
+    bool ok[Shape<U>::kGroups32];
+    groups_ok(lane, rest / 4, ok);
+    tile32(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint32_t *>(E.data) + begin) + lane, ok,
+           G0 + lane * 4, one, t0, t1);
+  } else {
+    bool ok[Shape<U>::kGroups16];
+    groups_ok(lane, rest / 8, ok);
+    tile16(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint16_t *>(E.data) + begin) + lane, ok,
+           G0 + lane * 8, one, t0, t1);
+  }
+  const uint64_t i = lane < 8 ? lane : E.head + body + (lane - 8);
+  if (i < (lane < 8 ? (uint64_t)E.head : E.n)) t0 += term<0>(E.key_base + (uint32_t)i, word_at(E, i), one);
+  return t0 + t1;
 }
 
 // Per-thread double buffering of full tiles in shared memory: while a thread
 // folds one tile it has the next one in flight with cp.async, into slots that
 // only it reads, so no barrier is needed; cp.async.wait_group orders each
 // thread's own copies.  Slot k of stage b of thread t is
-// stg[(b * kStageSlots + k) * kThreads + t]: a warp's 16-byte reads of one
-// slot are contiguous.
-constexpr int kStageSlots = 2 * kDigestUnroll;                       // 16-byte words per thread per stage
-constexpr uint32_t kStageBytes = 2u * kStageSlots * kThreads * 16u;  // two stages: 131,072 bytes
-constexpr uint32_t kLaunchSmem = kStageBytes + APC_DIGEST_EXTRA_SMEM;
+// stg[(b * slots + k) * kThreads + t]: a warp's 16-byte reads of one slot are
+// contiguous.  A stage has kGroups32 slots per thread.
+template <int U>
+constexpr uint32_t launch_smem() {  // two stages
+  return 2u * Shape<U>::kGroups32 * kThreads * 16u + APC_DIGEST_EXTRA_SMEM;
+}
+static_assert(launch_smem<kDigestLong>() <= 227 * 1024, "shared memory per CTA");
 
 __device__ __forceinline__ void cp16(uint32_t dst, const void *src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -158,15 +218,97 @@ __device__ __forceinline__ void flush(uint64_t &acc, int slot, unsigned long lon
   acc = 0;
 }
 
-__device__ __forceinline__ uint32_t word_at(const DigestEntry &E, uint64_t i) {
-  return E.dtype == 0 ? reinterpret_cast<const uint32_t *>(E.data)[i]
-                      : (uint32_t) reinterpret_cast<const uint16_t *>(E.data)[i];
+// The entry whose tiles hold `tile`, at or after entry `lo` (the last one that
+// begins at or before it: an entry without full tiles begins where the next
+// one does).
+template <int MAXE>
+__device__ __forceinline__ uint32_t entry_of(const DigestPlan<MAXE> &plan, uint32_t lo, uint64_t tile) {
+  uint32_t hi = plan.count;  // e[lo].tile_begin <= tile, e[hi] beyond
+  while (hi - lo > 1) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (plan.e[mid].tile_begin <= tile) lo = mid;
+    else hi = mid;
+  }
+  return lo;
 }
 
-// One CTA per SM (32 warps, 128 KB of stages), which caps the kernel at 64
-// registers: a full tile's 16 terms per thread, without per-vector checks,
-// form one block that the compiler schedules within them.
-template <int MAXE>
+// One walk: the warps' tiles of the fp32 entries (T32) or of the bf16 entries.
+// Each kind's tiles are shared out over all CTAs on their own: a bf16 tile
+// costs less than an fp32 one, and a CTA with tiles of one kind only would
+// finish early or late.
+template <bool T32, int U, int MAXE>
+__device__ __forceinline__ void walk(const DigestPlan<MAXE> &plan, uint4 *stg, uint32_t stg_t, unsigned long long *s_acc) {
+  using S = Shape<U>;
+  constexpr int kGroups = T32 ? S::kGroups32 : S::kGroups16, kStageSlots = S::kGroups32;
+  constexpr uint64_t kStep = kWarps * S::kTile;  // elements from a warp's tile to its next
+  constexpr uint32_t kWords = T32 ? 4 : 8;  // of a group
+  constexpr uint32_t kKeySpan = T32 ? S::kKeySpan32 : S::kKeySpan16;
+  const uint32_t one = plan.one;
+  const uint64_t lo = T32 ? 0 : plan.tiles32, hi = T32 ? plan.tiles32 : plan.total_tiles;
+  // this CTA's contiguous run of the kind's tiles, walked by its warps:
+  // tile t_begin + r for r = warp, warp + 32, ... below len
+  // (the bf16 runs are dealt out from the last CTA on, so that the longer runs
+  // of both kinds fall on different CTAs)
+  const uint32_t c = T32 ? blockIdx.x : gridDim.x - 1 - blockIdx.x;
+  const uint64_t per = (hi - lo) / gridDim.x, rem = (hi - lo) % gridDim.x;
+  const uint64_t t_begin = lo + c * per + (c < rem ? c : rem);
+  const uint32_t len = (uint32_t)(per + (c < rem ? 1 : 0));  // 2^32 tiles are 2^41 elements
+  int slot = -1;
+  uint64_t acc = 0;
+  uint32_t r = threadIdx.x >> 5, cur = 0;
+  while (r < len) {
+    cur = entry_of(plan, cur, t_begin + r);
+    const DigestEntry &E = plan.e[cur];
+    const uint64_t left = (cur + 1 < plan.count ? plan.e[cur + 1].tile_begin : plan.total_tiles) - t_begin;
+    const uint32_t stop = left < len ? (uint32_t)left : len;
+    if ((int)E.slot != slot) {
+      flush(acc, slot, s_acc);
+      slot = E.slot;
+    }
+    const uint64_t base = E.head + (t_begin + r - E.tile_begin) * S::kTile;  // the tile's first element
+    const uint32_t lane = threadIdx.x & 31;
+    const uint4 *q = reinterpret_cast<const uint4 *>(static_cast<const uint8_t *>(E.data) + base * (16 / kWords)) + lane;
+    uint32_t G0 = E.key_base + (uint32_t)base + lane * kWords;
+    uint64_t t0 = 0, t1 = 0;
+    uint32_t b = 0;
+    bool all[kGroups];
+#pragma unroll
+    for (int j = 0; j < kGroups; ++j) {
+      all[j] = true;  // a full tile needs no checks
+      cp16(stg_t + j * kThreads * 16u, q + j * 32);
+    }
+    cp_commit();
+    for (; r < stop; r += kWarps, q += kStep / kWords, G0 += (uint32_t)kStep) {
+      if (r + kWarps < stop) {
+        const uint4 *n = q + kStep / kWords;
+        const uint32_t dst = stg_t + (b ^ 1) * kStageSlots * kThreads * 16u;
+#pragma unroll
+        for (int j = 0; j < kGroups; ++j) cp16(dst + j * kThreads * 16u, n + j * 32);
+      }
+      cp_commit();
+      cp_wait_all_but_newest();
+      const uint4 *src = stg + b * kStageSlots * kThreads + threadIdx.x;
+      uint4 x[kGroups];
+#pragma unroll
+      for (int j = 0; j < kGroups; ++j) x[j] = src[j * kThreads];
+      const uint32_t B = G0 + 0x9E3779B9u;
+      const bool shared = top_bits_shared(B, kKeySpan);
+      if constexpr (T32) {
+        if (shared) fold32<true>(x, all, G0, one, B >> 30, t0, t1);
+        else fold32<false>(x, all, G0, one, 0, t0, t1);
+      } else {
+        if (shared) fold16<true>(x, all, G0, one, B >> 30, t0, t1);
+        else fold16<false>(x, all, G0, one, 0, t0, t1);
+      }
+      b ^= 1;
+    }
+    acc_add(acc, t0, one);
+    acc_add(acc, t1, one);
+  }
+  flush(acc, slot, s_acc);
+}
+
+template <int MAXE, int U>
 __global__ void __launch_bounds__(kThreads, APC_DIGEST_MIN_BLOCKS) digest_kernel(const __grid_constant__ DigestPlan<MAXE> plan,
                                                           unsigned long long *out) {
   __shared__ unsigned long long s_acc[APC_MAX_SLOTS];
@@ -174,124 +316,20 @@ __global__ void __launch_bounds__(kThreads, APC_DIGEST_MIN_BLOCKS) digest_kernel
   const uint32_t stg_t = (uint32_t)__cvta_generic_to_shared(stg + threadIdx.x);  // this thread's slot 0, stage 0
   if (threadIdx.x < APC_MAX_SLOTS) s_acc[threadIdx.x] = 0;
   __syncthreads();
-  const uint32_t one = plan.one;
-  int slot = -1;
-  uint64_t acc = 0;
-  // this CTA's contiguous run of the launch's tiles: [tile, t_end)
-  const uint64_t per = plan.total_tiles / gridDim.x, rem = plan.total_tiles % gridDim.x;
-  uint64_t tile = blockIdx.x * per + (blockIdx.x < rem ? blockIdx.x : rem);
-  const uint64_t t_end = tile + per + (blockIdx.x < rem ? 1 : 0);
-  uint32_t cur = 0;
-  while (cur + 1 < plan.count && tile >= plan.e[cur + 1].tile_begin) ++cur;
-  const uint64_t t8 = (uint64_t)threadIdx.x * kVec;
-  for (; tile < t_end; ++cur) {
-    const DigestEntry &E = plan.e[cur];
-    const uint64_t stop_e = cur + 1 < plan.count ? plan.e[cur + 1].tile_begin : plan.total_tiles;
-    const uint64_t stop = stop_e < t_end ? stop_e : t_end;
-    if (tile >= stop) continue;
-    if ((int)E.slot != slot) {
-      flush(acc, slot, s_acc);
-      slot = E.slot;
-    }
-    const uint64_t head = E.head;
-    const uint64_t vec_end = head + ((E.n - head) & ~(uint64_t)(kVec - 1));
-    uint64_t base = head + (tile - E.tile_begin) * kDigestTile + t8;   // this thread's first element
-    uint32_t G0 = E.key_base + (uint32_t)base;
-    const bool first = tile == E.tile_begin;
-    uint64_t t0 = 0, t1 = 0;
-    // Every tile of an entry but its last is full (all vectors of all threads
-    // lie in the body) and runs without per-vector checks.
-    const uint64_t full_end = stop_e - 1 < stop ? stop_e - 1 : stop;
-    bool all[kDigestUnroll], ok[kDigestUnroll];
-#pragma unroll
-    for (int u = 0; u < kDigestUnroll; ++u) all[u] = true;
-    if (E.dtype == 0) {
-      const uint32_t *d = reinterpret_cast<const uint32_t *>(E.data);
-      const uint4 *q = reinterpret_cast<const uint4 *>(d + base);
-      if (tile < full_end) {
-        uint32_t b = 0;
-#pragma unroll
-        for (int k = 0; k < kStageSlots; ++k) cp16(stg_t + k * kThreads * 16u, q + (k >> 1) * 2 * kThreads + (k & 1));
-        cp_commit();
-        for (; tile < full_end; ++tile, q += kDigestTile / 4, G0 += (uint32_t)kDigestTile) {
-          if (tile + 1 < full_end) {
-            const uint4 *n = q + kDigestTile / 4;
-            const uint32_t dst = stg_t + (b ^ 1) * kStageSlots * kThreads * 16u;
-#pragma unroll
-            for (int k = 0; k < kStageSlots; ++k) cp16(dst + k * kThreads * 16u, n + (k >> 1) * 2 * kThreads + (k & 1));
-          }
-          cp_commit();
-          cp_wait_all_but_newest();
-          const uint4 *src = stg + b * kStageSlots * kThreads + threadIdx.x;
-          uint4 x[kDigestUnroll][2];
-#pragma unroll
-          for (int u = 0; u < kDigestUnroll; ++u) {
-            x[u][0] = src[(2 * u) * kThreads];
-            x[u][1] = src[(2 * u + 1) * kThreads];
-          }
-          const uint32_t B = G0 + 0x9E3779B9u;
-          if (top_bits_shared(B, kTileKeySpan)) fold32<true>(x, all, G0, one, B >> 30, t0, t1);
-          else fold32<false>(x, all, G0, one, 0, t0, t1);
-          b ^= 1;
-        }
-      }
-      if (tile < stop) {  // the entry's last tile
-        last_tile_ok((uint64_t)(reinterpret_cast<const uint32_t *>(q) - d), vec_end, ok);
-        tile32(q, ok, G0, one, t0, t1);
-        ++tile;
-      }
-    } else {
-      const uint16_t *d = reinterpret_cast<const uint16_t *>(E.data);
-      const uint4 *q = reinterpret_cast<const uint4 *>(d + base);
-      if (tile < full_end) {
-        uint32_t b = 0;
-#pragma unroll
-        for (int u = 0; u < kDigestUnroll; ++u) cp16(stg_t + u * kThreads * 16u, q + u * kThreads);
-        cp_commit();
-        for (; tile < full_end; ++tile, q += kDigestTile / 8, G0 += (uint32_t)kDigestTile) {
-          if (tile + 1 < full_end) {
-            const uint4 *n = q + kDigestTile / 8;
-            const uint32_t dst = stg_t + (b ^ 1) * kStageSlots * kThreads * 16u;
-#pragma unroll
-            for (int u = 0; u < kDigestUnroll; ++u) cp16(dst + u * kThreads * 16u, n + u * kThreads);
-          }
-          cp_commit();
-          cp_wait_all_but_newest();
-          const uint4 *src = stg + b * kStageSlots * kThreads + threadIdx.x;
-          uint4 x[kDigestUnroll];
-#pragma unroll
-          for (int u = 0; u < kDigestUnroll; ++u) x[u] = src[u * kThreads];
-          const uint32_t B = G0 + 0x9E3779B9u;
-          if (top_bits_shared(B, kTileKeySpan)) fold16<true>(x, all, G0, one, B >> 30, t0, t1);
-          else fold16<false>(x, all, G0, one, 0, t0, t1);
-          b ^= 1;
-        }
-      }
-      if (tile < stop) {  // the entry's last tile
-        last_tile_ok((uint64_t)(reinterpret_cast<const uint16_t *>(q) - d), vec_end, ok);
-        tile16(q, ok, G0, one, t0, t1);
-        ++tile;
-      }
-    }
-    if (first) {   // the CTA that owns an entry's first tile also does its scalar head and tail
-      const uint32_t t = threadIdx.x;
-      if (t < head) { acc_add(t0, term<0>(E.key_base + t, word_at(E, t), one), one); }
-      if (t >= 32 && t - 32 < E.n - vec_end) {
-        const uint64_t i = vec_end + (t - 32);
-        acc_add(t0, term<0>(E.key_base + (uint32_t)i, word_at(E, i), one), one);
-      }
-    }
-    acc_add(acc, t0, one);
-    acc_add(acc, t1, one);
+  // what the entries hold beyond their full tiles, one entry per warp
+  for (uint32_t e = blockIdx.x + gridDim.x * (threadIdx.x >> 5); e < plan.count; e += gridDim.x * kWarps) {
+    uint64_t x = remainder<U>(plan.e[e], threadIdx.x & 31, plan.one);
+    flush(x, plan.e[e].slot, s_acc);
   }
-  flush(acc, slot, s_acc);
+  walk<true, U>(plan, stg, stg_t, s_acc);
+  walk<false, U>(plan, stg, stg_t, s_acc);
   __syncthreads();
   if (threadIdx.x < APC_MAX_SLOTS && s_acc[threadIdx.x]) atomicAdd(&out[threadIdx.x], s_acc[threadIdx.x]);
 }
 
 // The dynamic shared-memory limit of one instantiation, raised once per
 // device (later launches, for example inside a stream capture, only enqueue).
-template <int MAXE>
+template <int MAXE, int U>
 int ensure_stage_attribute() {
   static std::atomic<uint64_t> done_mask{0};
   int dev = 0;
@@ -299,41 +337,57 @@ int ensure_stage_attribute() {
   if (e != cudaSuccess) return (int)e;
   const uint64_t bit = dev < 64 ? (1ull << dev) : 0;
   if (bit && (done_mask.load(std::memory_order_acquire) & bit)) return 0;
-  e = cudaFuncSetAttribute(digest_kernel<MAXE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLaunchSmem);
+  e = cudaFuncSetAttribute(digest_kernel<MAXE, U>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)launch_smem<U>());
   if (e != cudaSuccess) return (int)e;
   if (APC_SMEM_CARVEOUT >= 0) {
-    e = cudaFuncSetAttribute(digest_kernel<MAXE>, cudaFuncAttributePreferredSharedMemoryCarveout, APC_SMEM_CARVEOUT);
+    e = cudaFuncSetAttribute(digest_kernel<MAXE, U>, cudaFuncAttributePreferredSharedMemoryCarveout, APC_SMEM_CARVEOUT);
     if (e != cudaSuccess) return (int)e;
   }
   if (bit) done_mask.fetch_or(bit, std::memory_order_acq_rel);
   return 0;
 }
 
-template <int MAXE>
-int launch_t(const DigestPlan<MAXE> &plan, unsigned grid, void *stream, unsigned long long *out) {
-  int e = ensure_stage_attribute<MAXE>();
+template <int MAXE, int U>
+int launch_u(const DigestPlan<MAXE> &plan, unsigned grid, void *stream, unsigned long long *out) {
+  int e = ensure_stage_attribute<MAXE, U>();
   if (e) return e;
-  digest_kernel<MAXE><<<grid, kThreads, kLaunchSmem, (cudaStream_t)stream>>>(plan, out);
+  digest_kernel<MAXE, U><<<grid, kThreads, launch_smem<U>(), (cudaStream_t)stream>>>(plan, out);
   return (int)cudaGetLastError();
 }
 
 template <int MAXE>
-int blocks_t(int *out) {
-  int e = ensure_stage_attribute<MAXE>();
+int launch_t(const DigestPlan<MAXE> &plan, int u, unsigned grid, void *stream, unsigned long long *out) {
+  return u == kDigestLong ? launch_u<MAXE, kDigestLong>(plan, grid, stream, out)
+                          : launch_u<MAXE, kDigestShort>(plan, grid, stream, out);
+}
+
+template <int MAXE, int U>
+int blocks_u(int *out) {
+  int e = ensure_stage_attribute<MAXE, U>();
   if (e) return e;
-  return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, digest_kernel<MAXE>, kThreads, kLaunchSmem);
+  return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, digest_kernel<MAXE, U>, kThreads, launch_smem<U>());
+}
+
+// One grid size serves both tile lengths: the smaller of their residencies.
+template <int MAXE>
+int blocks_t(int *out) {
+  int a = 0, b = 0;
+  int e = blocks_u<MAXE, kDigestShort>(&a);
+  if (e || (e = blocks_u<MAXE, kDigestLong>(&b))) return e;
+  *out = a < b ? a : b;
+  return 0;
 }
 
 }  // namespace
 
-int launch_digest_small(const DigestPlan<kDigestSmall> &plan, unsigned grid, void *stream,
+int launch_digest_small(const DigestPlan<kDigestSmall> &plan, int u, unsigned grid, void *stream,
                         unsigned long long *out) {
-  return launch_t<kDigestSmall>(plan, grid, stream, out);
+  return launch_t<kDigestSmall>(plan, u, grid, stream, out);
 }
 
-int launch_digest_large(const DigestPlan<kDigestLarge> &plan, unsigned grid, void *stream,
+int launch_digest_large(const DigestPlan<kDigestLarge> &plan, int u, unsigned grid, void *stream,
                         unsigned long long *out) {
-  return launch_t<kDigestLarge>(plan, grid, stream, out);
+  return launch_t<kDigestLarge>(plan, u, grid, stream, out);
 }
 
 int digest_blocks_per_sm(bool large, int *out) { return large ? blocks_t<kDigestLarge>(out) : blocks_t<kDigestSmall>(out); }

@@ -222,26 +222,30 @@ apc_status run_commit_batches(const std::vector<apc::CommitEntry> &entries, cons
   return APC_OK;
 }
 
-template <int MAXE, typename Launch>
-apc_status run_digest_batches(const std::vector<apc::DigestEntry> &entries, unsigned grid_cap, void *stream,
-                              unsigned long long *out, Launch launch, const char *what) {
+// Entries arrive with the element count of their vector body in tile_begin;
+// tiles_of(body) is the kernel's tile count of an entry.
+template <int MAXE, typename Tiles, typename Launch>
+apc_status run_digest_batches(const std::vector<apc::DigestEntry> &entries, unsigned grid_cap, Tiles tiles_of,
+                              Launch launch, const char *what) {
   auto plan = std::make_unique<apc::DigestPlan<MAXE>>();
   plan->one = 1;
   size_t i = 0;
   while (i < entries.size()) {
     const size_t k = std::min(entries.size() - i, (size_t)MAXE);
-    uint64_t tiles = 0;
+    uint64_t tiles = 0, tiles32 = 0;
     for (size_t j = 0; j < k; ++j) {
       apc::DigestEntry e = entries[i + j];
-      const uint64_t t = e.tile_begin;  // holds the entry's tile count until placed
+      const uint64_t t = tiles_of(e.tile_begin);
       e.tile_begin = tiles;
       tiles += t;
+      if (e.dtype == APC_F32) tiles32 = tiles;
       plan->e[j] = e;
     }
     plan->count = (uint32_t)k;
     plan->total_tiles = tiles;
-    const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(tiles, grid_cap));
-    int e = launch(*plan, grid, stream, out);
+    plan->tiles32 = tiles32;
+    const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(std::max<uint64_t>(tiles, k), grid_cap));
+    int e = launch(*plan, grid);
     if (e) return cuda_fail(e, what);
     i += k;
   }
@@ -392,21 +396,30 @@ APC_EXPORT apc_status apc_commit_step_bf16(const apc_tensor_bf16 *table, int32_t
 
 namespace {
 
-// Validate a buffer list and turn it into digest/count plan entries for a
-// kernel whose tiles hold `tile` elements.
+// Validate a buffer list and turn it into digest/count plan entries, ordered
+// by type, fp32 first, and inside a type by slot (a sum or a count does not
+// depend on the order): the digest kernel shares out each type's tiles on
+// their own, and a warp's walk over the plan seldom meets another slot and
+// flushes its running sum.
 apc_status buffer_entries(const apc_buffer *bufs, int32_t num_bufs, int32_t num_slots, uint64_t *out,
-                          uint64_t tile, std::vector<apc::DigestEntry> *entries) {
+                          std::vector<apc::DigestEntry> *entries) {
   if (num_bufs < 0) return fail(APC_EINVAL, "num_bufs %d < 0", num_bufs);
   if (num_bufs > 0 && !bufs) return fail(APC_EINVAL, "bufs pointer is null");
   if (num_slots < 1 || num_slots > APC_MAX_SLOTS)
     return fail(APC_EINVAL, "num_slots %d outside 1..%d", num_slots, APC_MAX_SLOTS);
   if (!out) return fail(APC_EINVAL, "output pointer is null");
   if ((uintptr_t)out % 8) return fail(APC_EALIGN, "output not 8-byte aligned");
-  entries->reserve((size_t)num_bufs);
   std::vector<Range> ranges;
   std::vector<Owned> owned;
   ranges.reserve((size_t)num_bufs + 1);
   owned.reserve((size_t)num_bufs + 1);
+  size_t at[2 * APC_MAX_SLOTS + 1] = {0};  // first entry of each (type, slot), then the next one to place
+  for (int32_t k = 0; k < num_bufs; ++k) {
+    const apc_buffer &b = bufs[k];
+    if (b.n && b.dtype <= APC_BF16 && b.slot < APC_MAX_SLOTS) ++at[b.dtype * APC_MAX_SLOTS + b.slot + 1];
+  }
+  for (int g = 0; g < 2 * APC_MAX_SLOTS; ++g) at[g + 1] += at[g];
+  entries->resize(at[2 * APC_MAX_SLOTS]);
   for (int32_t k = 0; k < num_bufs; ++k) {
     const apc_buffer &b = bufs[k];
     if (b.dtype != APC_F32 && b.dtype != APC_BF16) return fail(APC_EINVAL, "bufs[%d]: unknown dtype %u", k, b.dtype);
@@ -428,9 +441,8 @@ apc_status buffer_entries(const apc_buffer *bufs, int32_t num_bufs, int32_t num_
     e.dtype = (uint8_t)b.dtype;
     e.slot = (uint8_t)b.slot;
     e.pad_ = 0;
-    const uint64_t body = (b.n - e.head) / apc::kVec * apc::kVec;
-    e.tile_begin = std::max<uint64_t>(1, ceil_div(body, tile));  // tile count until placed
-    entries->push_back(e);
+    e.tile_begin = (b.n - e.head) / apc::kVec * apc::kVec;  // the vector body, until placed
+    (*entries)[at[b.dtype * APC_MAX_SLOTS + b.slot]++] = e;
   }
   const uintptr_t o = (uintptr_t)out;
   ranges.push_back({o, o + (uintptr_t)num_slots * sizeof(uint64_t), true});
@@ -445,7 +457,7 @@ APC_EXPORT apc_status apc_digest(const apc_buffer *bufs, int32_t num_bufs, int32
                                  uint64_t *out_digests) {
   g_last_error[0] = 0;
   std::vector<apc::DigestEntry> entries;
-  apc_status st = buffer_entries(bufs, num_bufs, num_slots, out_digests, apc::kDigestTile, &entries);
+  apc_status st = buffer_entries(bufs, num_bufs, num_slots, out_digests, &entries);
   if (st != APC_OK) return st;
   int e = (int)cudaMemsetAsync(out_digests, 0, (size_t)num_slots * sizeof(uint64_t), (cudaStream_t)stream);
   if (e) return cuda_fail(e, "cudaMemsetAsync(out_digests)");
@@ -453,18 +465,30 @@ APC_EXPORT apc_status apc_digest(const apc_buffer *bufs, int32_t num_bufs, int32
   Device d;
   if ((st = device_info(&d)) != APC_OK) return st;
   unsigned long long *out = reinterpret_cast<unsigned long long *>(out_digests);
-  if (entries.size() <= (size_t)apc::kDigestSmall)
-    return run_digest_batches<apc::kDigestSmall>(entries, grid_for(UINT64_MAX, d.sms, d.digest_small), stream, out,
-                                                 apc::launch_digest_small, "digest kernel launch");
-  return run_digest_batches<apc::kDigestLarge>(entries, grid_for(UINT64_MAX, d.sms, d.digest_large), stream, out,
-                                               apc::launch_digest_large, "digest kernel launch");
+  const bool small = entries.size() <= (size_t)apc::kDigestSmall;
+  const unsigned cap = grid_for(UINT64_MAX, d.sms, small ? d.digest_small : d.digest_large);
+  // long tiles where every warp of the grid gets several of them in a launch
+  uint64_t body = 0;
+  for (const apc::DigestEntry &en : entries) body += en.tile_begin;
+  const uint64_t warps = (uint64_t)cap * (apc::kThreads / 32);
+  const uint64_t launches = ceil_div(entries.size(), small ? apc::kDigestSmall : apc::kDigestLarge);
+  const int u = body / apc::digest_tile(apc::kDigestLong) >= apc::kDigestLongTiles * warps * launches ? apc::kDigestLong
+                                                                                                       : apc::kDigestShort;
+  const auto tiles_of = [u](uint64_t n) { return n / apc::digest_tile(u); };
+  if (small)
+    return run_digest_batches<apc::kDigestSmall>(
+        entries, cap, tiles_of, [&](const auto &plan, unsigned grid) { return apc::launch_digest_small(plan, u, grid, stream, out); },
+        "digest kernel launch");
+  return run_digest_batches<apc::kDigestLarge>(
+      entries, cap, tiles_of, [&](const auto &plan, unsigned grid) { return apc::launch_digest_large(plan, u, grid, stream, out); },
+      "digest kernel launch");
 }
 
 APC_EXPORT apc_status apc_count_nonzero(const apc_buffer *bufs, int32_t num_bufs, int32_t num_slots,
                                         apc_stream_t stream, uint64_t *out_counts) {
   g_last_error[0] = 0;
   std::vector<apc::DigestEntry> entries;
-  apc_status st = buffer_entries(bufs, num_bufs, num_slots, out_counts, apc::kCountTile, &entries);
+  apc_status st = buffer_entries(bufs, num_bufs, num_slots, out_counts, &entries);
   if (st != APC_OK) return st;
   int e = (int)cudaMemsetAsync(out_counts, 0, (size_t)num_slots * sizeof(uint64_t), (cudaStream_t)stream);
   if (e) return cuda_fail(e, "cudaMemsetAsync(out_counts)");
@@ -472,11 +496,16 @@ APC_EXPORT apc_status apc_count_nonzero(const apc_buffer *bufs, int32_t num_bufs
   Device d;
   if ((st = device_info(&d)) != APC_OK) return st;
   unsigned long long *out = reinterpret_cast<unsigned long long *>(out_counts);
+  const auto tiles_of = [](uint64_t n) { return std::max<uint64_t>(1, ceil_div(n, apc::kCountTile)); };
   if (entries.size() <= (size_t)apc::kDigestSmall)
-    return run_digest_batches<apc::kDigestSmall>(entries, grid_for(UINT64_MAX, d.sms, d.count_small), stream, out,
-                                                 apc::launch_count_small, "count kernel launch");
-  return run_digest_batches<apc::kDigestLarge>(entries, grid_for(UINT64_MAX, d.sms, d.count_large), stream, out,
-                                               apc::launch_count_large, "count kernel launch");
+    return run_digest_batches<apc::kDigestSmall>(
+        entries, grid_for(UINT64_MAX, d.sms, d.count_small), tiles_of,
+        [&](const auto &plan, unsigned grid) { return apc::launch_count_small(plan, grid, stream, out); },
+        "count kernel launch");
+  return run_digest_batches<apc::kDigestLarge>(
+      entries, grid_for(UINT64_MAX, d.sms, d.count_large), tiles_of,
+      [&](const auto &plan, unsigned grid) { return apc::launch_count_large(plan, grid, stream, out); },
+      "count kernel launch");
 }
 
 namespace {

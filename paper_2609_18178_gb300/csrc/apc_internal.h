@@ -137,20 +137,26 @@ static_assert(sizeof(CommitEntry) == 72, "entry layout");
 static_assert(sizeof(CommitPlan<kCommitLarge>) <= 32764, "kernel parameter limit");
 
 // Digest kernel: the loads are issued by the compute warps themselves (the
-// pass is bound by integer issue): a thread handles kDigestUnroll 8-element
-// vectors per tile.  One CTA of 1024 threads per SM puts 8 warps on each of
-// its four schedulers and gives each SM one contiguous run of tiles; two
-// CTAs of the same warps per SM run 2-3% slower, and shapes that load the
-// schedulers unevenly (11 or 13 warps per CTA) about 8% slower.
+// pass is bound by its integer pipes): a lane handles U 8-element vectors of
+// its warp's tile, whose terms form one block of independent work.  One CTA
+// per SM gives each SM one contiguous run of tiles.
+//  * 640 threads (5 warps on each of the four schedulers, 96 registers) with
+//    U = 4: 453 M elements of fp32 state verify in 1,427 us and 1.81 G of bf16
+//    state in 3,675 us, against 1,455 and 3,883 us for 1024 x 2, 1,430 and
+//    3,740 for 768 x 3, 1,452 and 3,879 for 512 x 4, 1,446 and 3,888 for
+//    640 x 5.
+//  * U = 4 needs several tiles for every warp to be dealt out evenly: with few
+//    of them a tile of half the length spreads the work better (1 M elements
+//    of fp32 state, 1.3 long tiles per warp: 9.9 us against 12.9).  The long
+//    tile is taken from kDigestLongTiles of them per warp on, where the last,
+//    partly dealt round costs at most 1 / 8 and typically half of that.
 #ifndef APC_DIGEST_THREADS
-#define APC_DIGEST_THREADS 1024
-#endif
-#ifndef APC_DIGEST_UNROLL
-#define APC_DIGEST_UNROLL 2
+#define APC_DIGEST_THREADS 640
 #endif
 constexpr int kThreads = APC_DIGEST_THREADS;     // threads per CTA of the digest kernel
-constexpr int kDigestUnroll = APC_DIGEST_UNROLL; // thread-vectors per thread per tile
-constexpr uint64_t kDigestTile = (uint64_t)kThreads * kVec * kDigestUnroll;  // 16,384 elements
+constexpr int kDigestShort = 2, kDigestLong = 4;  // U: vectors per lane per tile
+constexpr uint64_t kDigestLongTiles = 8;
+constexpr uint64_t digest_tile(int u) { return (uint64_t)32 * kVec * u; }  // elements: 512 and 1,024
 
 // Guard (count) kernel: the same plans and tiling scheme with its own shape;
 // one compare per word leaves it bound by HBM, so its shape is set by the
@@ -179,9 +185,9 @@ constexpr uint64_t kCountTile = (uint64_t)kCountThreads * kVec * kCountUnroll;  
 
 // One buffer of the digest kernel (32 bytes).
 //   head: scalar elements before the first 16-byte boundary (<= 7); then
-//         8-element vectors in tiles of kDigestTile (kCountTile for the
-//         count kernel); then a scalar tail, done
-//         by the CTA that owns the buffer's first tile.
+//         8-element vectors in tiles (digest_tile(U) elements, full ones
+//         only, for the digest kernel; kCountTile for the count kernel); then a
+//         scalar tail.
 struct DigestEntry {
   const void *data;
   uint64_t n;
@@ -196,6 +202,7 @@ struct DigestEntry {
 template <int MAXE>
 struct DigestPlan {
   uint64_t total_tiles;
+  uint64_t tiles32;      // tiles of the fp32 entries, which come first (digest kernel)
   uint32_t count;
   uint32_t one;          // 1: the FMA-pipe carry-add multiplier of the digest
   DigestEntry e[MAXE];
@@ -254,9 +261,9 @@ int launch_commit_small(const CommitPlan<kCommitSmall> &plan, int layout, bool z
                         void *stream, unsigned long long *out);
 int launch_commit_large(const CommitPlan<kCommitLarge> &plan, int layout, bool zero_grad, unsigned grid,
                         void *stream, unsigned long long *out);
-int launch_digest_small(const DigestPlan<kDigestSmall> &plan, unsigned grid, void *stream,
+int launch_digest_small(const DigestPlan<kDigestSmall> &plan, int u, unsigned grid, void *stream,
                         unsigned long long *out);
-int launch_digest_large(const DigestPlan<kDigestLarge> &plan, unsigned grid, void *stream,
+int launch_digest_large(const DigestPlan<kDigestLarge> &plan, int u, unsigned grid, void *stream,
                         unsigned long long *out);
 
 // Resident CTAs per SM of each kernel (cudaOccupancyMaxActiveBlocksPerMultiprocessor).

@@ -1,0 +1,99 @@
+"""Kernel paths chosen by a launch's sizes and alignments, at the sizes where
+each can go wrong, against the oracle.  The library's contract is exact bits,
+so every comparison is an equality."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2609_18178_gb300 as apc
+from apc_testlib import M64
+
+pytestmark = pytest.mark.gpu
+
+
+def grid_limit(monkeypatch, limit):
+    if limit is None:
+        monkeypatch.delenv("APC_GRID_LIMIT", raising=False)
+    else:
+        monkeypatch.setenv("APC_GRID_LIMIT", str(limit))
+
+
+def words(rng, n, f32):
+    if f32:
+        return rng.integers(0, 2**32, size=n, dtype=np.uint64).astype(np.uint32)
+    return rng.integers(0, 2**16, size=n, dtype=np.uint64).astype(np.uint16)
+
+
+def dev_words(a):
+    return torch.from_numpy(a.view(np.int32 if a.itemsize == 4 else np.int16)).cuda()
+
+
+def digest_of(a, goff):
+    return (oracle.digest_f32 if a.itemsize == 4 else oracle.digest_u16)(a, goff)
+
+
+# The verification kernel's warp tiles hold 512 elements, or 1,024 where every
+# warp of the grid gets at least 8 of those (on one CTA of 20 warps: from
+# 163,840 elements on).
+@pytest.mark.parametrize("limit,filler", [(None, 0), (1, 0), (1, 200_000), (3, 600_000)])
+def test_digest_warp_tiles(monkeypatch, limit, filler):
+    """Buffers of no, one and several warp tiles with every remainder of
+    vectors, head and tail, types and slots mixed, in short and long tiles
+    (the filler buffer's work selects the long ones)."""
+    grid_limit(monkeypatch, limit)
+    rng = np.random.default_rng(7)
+    sizes = [1, 5, 8, 17, 255, 256, 504] + [k * 512 + d for k in (1, 2, 3, 4, 41) for d in (-9, -8, -1, 0, 1, 8, 250, 264)]
+    bufs, want, keep = [], [0] * 8, []
+    for i, n in enumerate(sizes + ([filler] if filler else [])):
+        for f32 in (True, False):
+            shift = int(rng.integers(0, 8))
+            goff = int(rng.integers(0, 1 << 33))
+            a = words(rng, n + shift, f32)
+            slot = (3 * i + f32) % 8
+            want[slot] = (want[slot] + digest_of(a[shift:], goff)) & M64
+            keep.append(dev_words(a))
+            bufs.append(apc.BufferEntry(keep[-1][shift:], slot, goff, apc.F32 if f32 else apc.BF16))
+    assert apc.digests_to_host(apc.digest(bufs, 8)) == want
+    if not filler:   # each alone, so that no wrong term hides in a sum
+        for b, a in zip(bufs, keep):
+            ref = a.cpu().numpy()
+            ref = ref.view(np.uint32 if ref.itemsize == 4 else np.uint16)[ref.size - b.data.numel():]
+            one = apc.BufferEntry(b.data, 0, b.global_offset, b.dtype)
+            assert apc.digests_to_host(apc.digest([one], 1))[0] == digest_of(ref, b.global_offset)
+
+
+@pytest.mark.parametrize("limit", [None, 1])
+@pytest.mark.parametrize("f32", [True, False])
+def test_digest_tiles_across_top_bits(monkeypatch, f32, limit):
+    """Tiles whose incremented key high words cross a multiple of 2^30 (where
+    the shared top bits do not hold), short tiles and long ones."""
+    grid_limit(monkeypatch, limit)
+    rng = np.random.default_rng(11)
+    n = 200_003
+    a = words(rng, n, f32)
+    t = dev_words(a)
+    for q in range(4):
+        cross = (q * 2**30 - 0x9E3779B9) % 2**32
+        for back in (n - 5, 100_000, 1029, 3):
+            goff = (cross - back) % 2**32 + (2**32 if q == 2 else 0)
+            got = apc.digests_to_host(apc.digest([apc.BufferEntry(t, 0, goff, apc.F32 if f32 else apc.BF16)], 1))[0]
+            assert got == digest_of(a, goff), (q, back)
+
+
+def test_digest_many_short_buffers():
+    """More buffers than one launch holds, most without a full tile, slots and
+    types interleaved, some empty."""
+    rng = np.random.default_rng(13)
+    flat32, flat16 = words(rng, 700_000, True), words(rng, 700_000, False)
+    d32, d16 = dev_words(flat32), dev_words(flat16)
+    bufs, want, at = [], [0] * 5, 0
+    for i in range(2300):
+        n = int(rng.integers(0, 300)) if i % 97 else 3000 + i
+        f32 = bool(rng.integers(0, 2))
+        src, d = (flat32, d32) if f32 else (flat16, d16)
+        slot, goff = int(rng.integers(0, 5)), int(rng.integers(0, 1 << 34))
+        want[slot] = (want[slot] + digest_of(src[at:at + n], goff)) & M64
+        bufs.append(apc.BufferEntry(d[at:at + n], slot, goff, apc.F32 if f32 else apc.BF16))
+        at += n
+    assert apc.digests_to_host(apc.digest(bufs, 5)) == want
