@@ -75,9 +75,7 @@ __device__ __forceinline__ float bf16_value(uint32_t h) { return __uint_as_float
 // Two binary32 values rounded to bf16 (nearest even) by one paired
 // conversion, `lo` in the low half: each half equals bf16_rne_bits of its
 // input for every non-NaN value.
-// The bf16 layout rounds its three outputs this way, in pairs of elements
-// (2.5% faster there); for the fp32 layout's single w per element pairing
-// measured 0.2% slower, so it keeps one conversion per element.
+// The digest takes each half straight from the pair (hterm).
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t *>(&h);
@@ -113,12 +111,13 @@ __device__ __forceinline__ uint64_t cterm(uint32_t G, uint32_t bits, uint32_t on
   else return digest_term<K>(G, bits, one);
 }
 
-// The term of a 16-bit word (w, and the bf16 layout's p', m', v'): with the
-// shared top bits, the 16-bit form digest_term_u16.
-template <uint32_t K, bool SHARED>
-__device__ __forceinline__ uint64_t hterm(uint32_t G, uint32_t bits, uint32_t one, uint32_t top) {
-  if constexpr (SHARED) return digest_term_u16<K>(G, bits, one, top);
-  else return digest_term<K>(G, bits, one);
+// The term of half HALF (0 low, 1 high) of a packed pair of 16-bit words (w,
+// and the bf16 layout's p', m', v'): with the shared top bits, the 16-bit form
+// that takes the half by a dot product.
+template <uint32_t K, int HALF, bool SHARED>
+__device__ __forceinline__ uint64_t hterm(uint32_t G, uint32_t pair, uint32_t one, uint32_t top) {
+  if constexpr (SHARED) return digest_term_half<K, HALF>(G, pair, one, top);
+  else return digest_term<K>(G, HALF ? pair >> 16 : pair & 0xFFFFu, one);
 }
 
 // ------------------------------------------------------------ fp32 state
@@ -154,41 +153,42 @@ struct F32State {
     float m[4] = {r.m.x, r.m.y, r.m.z, r.m.w};
     float v[4] = {r.v.x, r.v.y, r.v.z, r.v.w};
     const uint32_t gw[4] = {r.g.x & 0xFFFFu, r.g.x >> 16, r.g.y & 0xFFFFu, r.g.y >> 16};
-    uint32_t w[4];
     if constexpr (PAIRED) {
-      adamw_pair(p[0], p[1], m[0], m[1], v[0], v[1], gw[0], gw[1], s, w[0], w[1]);
-      adamw_pair(p[2], p[3], m[2], m[3], v[2], v[3], gw[2], gw[3], s, w[2], w[3]);
+      uint32_t unused[4];
+      adamw_pair(p[0], p[1], m[0], m[1], v[0], v[1], gw[0], gw[1], s, unused[0], unused[1]);
+      adamw_pair(p[2], p[3], m[2], m[3], v[2], v[3], gw[2], gw[3], s, unused[2], unused[3]);
     } else {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) w[j] = adamw_element(p[j], m[j], v[j], gw[j], s);
+      for (int j = 0; j < 4; ++j) (void)adamw_element(p[j], m[j], v[j], gw[j], s);
     }
     __stcs(reinterpret_cast<float4 *>(static_cast<float *>(d.p) + off), make_float4(p[0], p[1], p[2], p[3]));
     __stcs(reinterpret_cast<float4 *>(static_cast<float *>(d.m) + off), make_float4(m[0], m[1], m[2], m[3]));
     __stcs(reinterpret_cast<float4 *>(static_cast<float *>(d.v) + off), make_float4(v[0], v[1], v[2], v[3]));
-    __stcs(reinterpret_cast<uint2 *>(d.w + off), make_uint2(w[0] | (w[1] << 16), w[2] | (w[3] << 16)));
+    const uint32_t w01 = pack_bf16x2(p[0], p[1]), w23 = pack_bf16x2(p[2], p[3]);
+    __stcs(reinterpret_cast<uint2 *>(d.w + off), make_uint2(w01, w23));
     // the group's keys are G + OFF .. G + OFF + 3
     const uint32_t B = G + (0x9E3779B9u + OFF);
     const uint32_t pb[4] = {__float_as_uint(p[0]), __float_as_uint(p[1]), __float_as_uint(p[2]), __float_as_uint(p[3])};
     const uint32_t mb[4] = {__float_as_uint(m[0]), __float_as_uint(m[1]), __float_as_uint(m[2]), __float_as_uint(m[3])};
     const uint32_t vb[4] = {__float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]), __float_as_uint(v[3])};
     if (top_bits_shared(B, 4)) {
-      fold<OFF, true>(G, pb, mb, vb, w, s.one, B >> 30, a);
+      fold<OFF, true>(G, pb, mb, vb, w01, w23, s.one, B >> 30, a);
     } else {
-      fold<OFF, false>(G, pb, mb, vb, w, s.one, 0, a);
+      fold<OFF, false>(G, pb, mb, vb, w01, w23, s.one, 0, a);
     }
   }
 
   template <uint32_t OFF, bool SHARED>
   __device__ static void fold(uint32_t G, const uint32_t (&p)[4], const uint32_t (&m)[4], const uint32_t (&v)[4],
-                              const uint32_t (&w)[4], uint32_t one, uint32_t top, Acc &a) {
+                              uint32_t w01, uint32_t w23, uint32_t one, uint32_t top, Acc &a) {
     a.p += cterm<OFF, SHARED>(G, p[0], one, top) + cterm<OFF + 1, SHARED>(G, p[1], one, top);
     a.p += cterm<OFF + 2, SHARED>(G, p[2], one, top) + cterm<OFF + 3, SHARED>(G, p[3], one, top);
     a.m += cterm<OFF, SHARED>(G, m[0], one, top) + cterm<OFF + 1, SHARED>(G, m[1], one, top);
     a.m += cterm<OFF + 2, SHARED>(G, m[2], one, top) + cterm<OFF + 3, SHARED>(G, m[3], one, top);
     a.v += cterm<OFF, SHARED>(G, v[0], one, top) + cterm<OFF + 1, SHARED>(G, v[1], one, top);
     a.v += cterm<OFF + 2, SHARED>(G, v[2], one, top) + cterm<OFF + 3, SHARED>(G, v[3], one, top);
-    a.w += hterm<OFF, SHARED>(G, w[0], one, top) + hterm<OFF + 1, SHARED>(G, w[1], one, top);
-    a.w += hterm<OFF + 2, SHARED>(G, w[2], one, top) + hterm<OFF + 3, SHARED>(G, w[3], one, top);
+    a.w += hterm<OFF, 0, SHARED>(G, w01, one, top) + hterm<OFF + 1, 1, SHARED>(G, w01, one, top);
+    a.w += hterm<OFF + 2, 0, SHARED>(G, w23, one, top) + hterm<OFF + 3, 1, SHARED>(G, w23, one, top);
   }
 
   __device__ static void one(const CommitEntry &E, uint64_t i, const Scalars &s, Acc &a) {
@@ -263,26 +263,21 @@ struct BF16State {
     __stcs(reinterpret_cast<uint2 *>(static_cast<uint16_t *>(d.p) + off), make_uint2(p01, p23));
     __stcs(reinterpret_cast<uint2 *>(static_cast<uint16_t *>(d.m) + off), make_uint2(m01, m23));
     __stcs(reinterpret_cast<uint2 *>(static_cast<uint16_t *>(d.v) + off), make_uint2(v01, v23));
-    const uint32_t po[4] = {p01 & 0xFFFFu, p01 >> 16, p23 & 0xFFFFu, p23 >> 16};
-    const uint32_t mo[4] = {m01 & 0xFFFFu, m01 >> 16, m23 & 0xFFFFu, m23 >> 16};
-    const uint32_t vo[4] = {v01 & 0xFFFFu, v01 >> 16, v23 & 0xFFFFu, v23 >> 16};
     const uint32_t B = G + (0x9E3779B9u + OFF);  // the group's keys are G + OFF .. G + OFF + 3
     if (top_bits_shared(B, 4)) {
-      fold<OFF, true>(G, po, mo, vo, s.one, B >> 30, a);
+      fold2<OFF, true>(G, p01, m01, v01, s.one, B >> 30, a);
+      fold2<OFF + 2, true>(G, p23, m23, v23, s.one, B >> 30, a);
     } else {
-      fold<OFF, false>(G, po, mo, vo, s.one, 0, a);
+      fold2<OFF, false>(G, p01, m01, v01, s.one, 0, a);
+      fold2<OFF + 2, false>(G, p23, m23, v23, s.one, 0, a);
     }
   }
 
-  template <uint32_t OFF, bool SHARED>
-  __device__ static void fold(uint32_t G, const uint32_t (&p)[4], const uint32_t (&m)[4], const uint32_t (&v)[4],
-                              uint32_t one, uint32_t top, Acc &a) {
-    a.p += hterm<OFF, SHARED>(G, p[0], one, top) + hterm<OFF + 1, SHARED>(G, p[1], one, top);
-    a.p += hterm<OFF + 2, SHARED>(G, p[2], one, top) + hterm<OFF + 3, SHARED>(G, p[3], one, top);
-    a.m += hterm<OFF, SHARED>(G, m[0], one, top) + hterm<OFF + 1, SHARED>(G, m[1], one, top);
-    a.m += hterm<OFF + 2, SHARED>(G, m[2], one, top) + hterm<OFF + 3, SHARED>(G, m[3], one, top);
-    a.v += hterm<OFF, SHARED>(G, v[0], one, top) + hterm<OFF + 1, SHARED>(G, v[1], one, top);
-    a.v += hterm<OFF + 2, SHARED>(G, v[2], one, top) + hterm<OFF + 3, SHARED>(G, v[3], one, top);
+  template <uint32_t K, bool SHARED>
+  __device__ __forceinline__ static void fold2(uint32_t G, uint32_t p, uint32_t m, uint32_t v, uint32_t one, uint32_t top, Acc &a) {
+    a.p += hterm<K, 0, SHARED>(G, p, one, top) + hterm<K + 1, 1, SHARED>(G, p, one, top);
+    a.m += hterm<K, 0, SHARED>(G, m, one, top) + hterm<K + 1, 1, SHARED>(G, m, one, top);
+    a.v += hterm<K, 0, SHARED>(G, v, one, top) + hterm<K + 1, 1, SHARED>(G, v, one, top);
   }
 
   __device__ static void one(const CommitEntry &E, uint64_t i, const Scalars &s, Acc &a) {
