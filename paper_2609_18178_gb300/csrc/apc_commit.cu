@@ -30,10 +30,20 @@
 //    the global stores are contiguous across the warp), release the
 //    stage to the producer, then apply AdamW, store the results with
 //    streaming stores, and fold the digest terms into 64-bit registers.
-//  * Elements outside the aligned bodies (entry heads and tails under 8
-//    elements, and entries whose buffers are not mutually 16-byte aligned)
-//    are "scalar items", done afterwards by the consumers with a grid-stride
-//    loop straight from global memory.
+//  * Entries whose buffers are not mutually 16-byte aligned (a packed flat
+//    shard of odd-sized tensors beside gradients and copies with boundaries of
+//    their own) run through the same ring: the producer copies, for each
+//    buffer, the 16-byte blocks that hold the tile, and the consumers read
+//    the words at the buffers' own offsets, lane-consecutive, and store them
+//    one by one.  That keeps whole tiles in flight where element loads straight
+//    from global memory kept one element per thread: 60 M elements in 291 odd
+//    entries take 386 us (606 before, 247 at the copy rate).  Tables without
+//    such an entry run an instantiation without this code (MIS = false).
+//  * What lies outside the tiles (fewer than 8 elements at each end of an
+//    aligned entry, at most 8 and 15 of a misaligned one, whole entries under
+//    32 elements of the latter) is done straight from global memory by the
+//    producer warp once it has issued its copies, so that it costs the
+//    consumers nothing.
 //  * At exit the CTA sums each digest (warp shuffles, shared memory) and adds
 //    it into the caller's output with one 64-bit atomic; addition mod 2^64 is
 //    order-free, so digests do not depend on grid size or table split.
@@ -74,8 +84,8 @@ __device__ __forceinline__ float bf16_value(uint32_t h) { return __uint_as_float
 
 // Two binary32 values rounded to bf16 (nearest even) by one paired
 // conversion, `lo` in the low half: each half equals bf16_rne_bits of its
-// input for every non-NaN value.
-// The digest takes each half straight from the pair (hterm).
+// input for every non-NaN value.  The digest takes each half straight from
+// the pair (hterm).
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t *>(&h);
@@ -95,11 +105,16 @@ struct Dst {
 // makes it visible to them): the addresses of the tile's first element in
 // p, m, v, w and g, its element count and its first digest index.  The
 // consumers then spend no instructions locating the tile in the chunk table.
+// A misaligned tile's cnt also holds kMisTile and, from bit 16 on, four bits
+// each: the byte offsets of its first element in the staged blocks of p, m, v
+// and g.
 struct __align__(16) StageDesc {
   uint8_t *p, *m, *v;
   uint16_t *w, *g;
   uint32_t cnt, G;
 };
+constexpr uint32_t kMisTile = 1u << 15;
+static_assert(kCommitTile < kMisTile && kCommitTileBF16 < kMisTile, "a tile's count and kMisTile share a word");
 static_assert(sizeof(StageDesc) == 48, "three 16-byte shared-memory loads");
 
 // A commit digest term.  With SHARED the caller has established that the
@@ -132,16 +147,68 @@ struct F32State {
   static constexpr int kBoundThreads = kThreads > APC_COMMIT_BOUND_THREADS ? kThreads : APC_COMMIT_BOUND_THREADS;
   static constexpr int kGroups = kCommitGroups;
   static constexpr uint64_t kTile = kCommitTile;
+  static constexpr int kMisUnroll = 2;      // pairs of a misaligned tile at a time
   struct Regs {
     float4 p, m, v;
     uint2 g;
   };
 
+  // PAD: bytes between the stage's regions (16 where misaligned tiles may come).
+  template <uint32_t PAD>
   __device__ static void load(const uint8_t *st, uint32_t e, Regs &r) {
     r.p = *reinterpret_cast<const float4 *>(st + 4 * e);
-    r.m = *reinterpret_cast<const float4 *>(st + 4 * (kTile + e));
-    r.v = *reinterpret_cast<const float4 *>(st + 4 * (2 * kTile + e));
-    r.g = *reinterpret_cast<const uint2 *>(st + 12 * kTile + 2 * e);
+    r.m = *reinterpret_cast<const float4 *>(st + 4 * (kTile + e) + PAD);
+    r.v = *reinterpret_cast<const float4 *>(st + 4 * (2 * kTile + e) + 2 * PAD);
+    r.g = *reinterpret_cast<const uint2 *>(st + 12 * kTile + 2 * e + 3 * PAD);
+  }
+
+  // Where a misaligned tile's elements sit in its stage.
+  struct Mis {
+    const float *p, *m, *v;
+    const uint16_t *g;
+    __device__ Mis(const uint8_t *st, uint32_t cnt) {
+      p = reinterpret_cast<const float *>(st + (cnt >> 16 & 15));
+      m = reinterpret_cast<const float *>(st + 4 * kTile + 16 + (cnt >> 20 & 15));
+      v = reinterpret_cast<const float *>(st + 8 * kTile + 32 + (cnt >> 24 & 15));
+      g = reinterpret_cast<const uint16_t *>(st + 12 * kTile + 48 + (cnt >> 28));
+    }
+  };
+
+  // Elements e and e + kConsumers of a misaligned tile.
+  template <bool ZERO>
+  __device__ static void mis_pair(const StageDesc &sd, const Mis &x, uint32_t e, const Scalars &s, Acc &a) {
+    const uint32_t f = e + kConsumers;
+    float p0 = x.p[e], p1 = x.p[f], m0 = x.m[e], m1 = x.m[f], v0 = x.v[e], v1 = x.v[f];
+    uint32_t w0, w1;
+    adamw_pair(p0, p1, m0, m1, v0, v1, x.g[e], x.g[f], s, w0, w1);
+    mis_store<ZERO>(sd, e, p0, m0, v0, w0);
+    mis_store<ZERO>(sd, f, p1, m1, v1, w1);
+    const uint32_t G = sd.G + e;
+    a.p += digest_term<0>(G, __float_as_uint(p0), s.one) + digest_term<kConsumers>(G, __float_as_uint(p1), s.one);
+    a.m += digest_term<0>(G, __float_as_uint(m0), s.one) + digest_term<kConsumers>(G, __float_as_uint(m1), s.one);
+    a.v += digest_term<0>(G, __float_as_uint(v0), s.one) + digest_term<kConsumers>(G, __float_as_uint(v1), s.one);
+    a.w += digest_term<0>(G, w0, s.one) + digest_term<kConsumers>(G, w1, s.one);
+  }
+
+  // Element e of a misaligned tile.
+  template <bool ZERO>
+  __device__ static void mis_one(const StageDesc &sd, const Mis &x, uint32_t e, const Scalars &s, Acc &a) {
+    float p = x.p[e], m = x.m[e], v = x.v[e];
+    const uint32_t w = adamw_element(p, m, v, x.g[e], s), G = sd.G + e;
+    mis_store<ZERO>(sd, e, p, m, v, w);
+    acc_add(a.p, digest_term(G, __float_as_uint(p), s.one), s.one);
+    acc_add(a.m, digest_term(G, __float_as_uint(m), s.one), s.one);
+    acc_add(a.v, digest_term(G, __float_as_uint(v), s.one), s.one);
+    acc_add(a.w, digest_term(G, w, s.one), s.one);
+  }
+
+  template <bool ZERO>
+  __device__ __forceinline__ static void mis_store(const StageDesc &sd, uint32_t e, float p, float m, float v, uint32_t w) {
+    __stcs(reinterpret_cast<float *>(sd.p) + e, p);
+    __stcs(reinterpret_cast<float *>(sd.m) + e, m);
+    __stcs(reinterpret_cast<float *>(sd.v) + e, v);
+    __stcs(sd.w + e, (uint16_t)w);
+    if (ZERO) __stcs(sd.g + e, (uint16_t)0);
   }
 
   // Four consecutive elements at the compile-time element offset OFF from
@@ -219,15 +286,62 @@ struct BF16State {
   static constexpr int kBoundThreads = kThreads;
   static constexpr int kGroups = kCommitGroupsBF16;
   static constexpr uint64_t kTile = kCommitTileBF16;
+  static constexpr int kMisUnroll = 1;      // two spill at 72 registers
   struct Regs {
     uint2 p, m, v, g;
   };
 
+  template <uint32_t PAD>
   __device__ static void load(const uint8_t *st, uint32_t e, Regs &r) {
     r.p = *reinterpret_cast<const uint2 *>(st + 2 * e);
-    r.m = *reinterpret_cast<const uint2 *>(st + 2 * (kTile + e));
-    r.v = *reinterpret_cast<const uint2 *>(st + 2 * (2 * kTile + e));
-    r.g = *reinterpret_cast<const uint2 *>(st + 6 * kTile + 2 * e);
+    r.m = *reinterpret_cast<const uint2 *>(st + 2 * (kTile + e) + PAD);
+    r.v = *reinterpret_cast<const uint2 *>(st + 2 * (2 * kTile + e) + 2 * PAD);
+    r.g = *reinterpret_cast<const uint2 *>(st + 6 * kTile + 2 * e + 3 * PAD);
+  }
+
+  struct Mis {
+    const uint16_t *p, *m, *v, *g;
+    __device__ Mis(const uint8_t *st, uint32_t cnt) {
+      p = reinterpret_cast<const uint16_t *>(st + (cnt >> 16 & 15));
+      m = reinterpret_cast<const uint16_t *>(st + 2 * kTile + 16 + (cnt >> 20 & 15));
+      v = reinterpret_cast<const uint16_t *>(st + 4 * kTile + 32 + (cnt >> 24 & 15));
+      g = reinterpret_cast<const uint16_t *>(st + 6 * kTile + 48 + (cnt >> 28));
+    }
+  };
+
+  template <bool ZERO>
+  __device__ static void mis_pair(const StageDesc &sd, const Mis &x, uint32_t e, const Scalars &s, Acc &a) {
+    const uint32_t f = e + kConsumers;
+    float p0 = bf16_value(x.p[e]), p1 = bf16_value(x.p[f]), m0 = bf16_value(x.m[e]), m1 = bf16_value(x.m[f]);
+    float v0 = bf16_value(x.v[e]), v1 = bf16_value(x.v[f]);
+    uint32_t unused0, unused1;
+    adamw_pair(p0, p1, m0, m1, v0, v1, x.g[e], x.g[f], s, unused0, unused1);
+    const uint32_t p = pack_bf16x2(p0, p1), m = pack_bf16x2(m0, m1), v = pack_bf16x2(v0, v1);
+    mis_store<ZERO>(sd, e, p & 0xFFFFu, m & 0xFFFFu, v & 0xFFFFu);
+    mis_store<ZERO>(sd, f, p >> 16, m >> 16, v >> 16);
+    const uint32_t G = sd.G + e;
+    a.p += digest_term<0>(G, p & 0xFFFFu, s.one) + digest_term<kConsumers>(G, p >> 16, s.one);
+    a.m += digest_term<0>(G, m & 0xFFFFu, s.one) + digest_term<kConsumers>(G, m >> 16, s.one);
+    a.v += digest_term<0>(G, v & 0xFFFFu, s.one) + digest_term<kConsumers>(G, v >> 16, s.one);
+  }
+
+  template <bool ZERO>
+  __device__ static void mis_one(const StageDesc &sd, const Mis &x, uint32_t e, const Scalars &s, Acc &a) {
+    float p = bf16_value(x.p[e]), m = bf16_value(x.m[e]), v = bf16_value(x.v[e]);
+    const uint32_t po = adamw_element(p, m, v, x.g[e], s), mo = bf16_rne_bits(m), vo = bf16_rne_bits(v);
+    mis_store<ZERO>(sd, e, po, mo, vo);
+    const uint32_t G = sd.G + e;
+    acc_add(a.p, digest_term(G, po, s.one), s.one);
+    acc_add(a.m, digest_term(G, mo, s.one), s.one);
+    acc_add(a.v, digest_term(G, vo, s.one), s.one);
+  }
+
+  template <bool ZERO>
+  __device__ __forceinline__ static void mis_store(const StageDesc &sd, uint32_t e, uint32_t p, uint32_t m, uint32_t v) {
+    __stcs(reinterpret_cast<uint16_t *>(sd.p) + e, (uint16_t)p);
+    __stcs(reinterpret_cast<uint16_t *>(sd.m) + e, (uint16_t)m);
+    __stcs(reinterpret_cast<uint16_t *>(sd.v) + e, (uint16_t)v);
+    if (ZERO) __stcs(sd.g + e, (uint16_t)0);
   }
 
   template <uint32_t OFF, bool PAIRED>
@@ -313,17 +427,27 @@ __device__ __forceinline__ void store_groups(const Dst &d, uint32_t G1, const ty
   if constexpr (K + 1 < L::kGroups) store_groups<L, ZERO, K + 1>(d, G1, r, ok, s, a);
 }
 
-template <class L>
+// The stage's four regions; with MIS each has 16 bytes more, for the blocks
+// that a misaligned tile begins and ends in.
+template <class L, bool MIS>
 __host__ __device__ constexpr uint32_t stage_bytes() {
-  return (uint32_t)L::kTile * (3 * L::kES + 2);
+  return (uint32_t)L::kTile * (3 * L::kES + 2) + (MIS ? 64 : 0);
 }
 
-template <class L>
+template <class L, bool MIS>
 __host__ __device__ constexpr uint32_t smem_bytes() {
-  return (uint32_t)L::kStages * stage_bytes<L>();
+  return (uint32_t)L::kStages * stage_bytes<L, MIS>();
 }
+static_assert(smem_bytes<F32State, true>() <= 226 * 1024 && smem_bytes<BF16State, true>() <= 226 * 1024,
+              "shared memory per CTA");
 
-static_assert(smem_bytes<F32State>() <= 227 * 1024 && smem_bytes<BF16State>() <= 227 * 1024, "shared memory per CTA");
+// Copy the 16-byte blocks that hold `bytes` bytes from `src` on into the
+// region at `dst`; the offset of the first byte in it is src % 16.
+__device__ __forceinline__ void copy_blocks(uint8_t *dst, const uint8_t *src, uint32_t bytes, uint64_t *bar,
+                                            uint64_t policy) {
+  const uint32_t off = (uint32_t)((uintptr_t)src & 15);
+  bulk_g2s(dst, src - off, (off + bytes + 15) & ~15u, bar, policy);
+}
 
 template <int MAXE>
 __device__ __forceinline__ uint32_t find_tile(const CommitPlan<MAXE> &plan, uint32_t cur, uint64_t tile) {
@@ -346,9 +470,10 @@ __device__ __forceinline__ TileWalk tile_walk(uint64_t total) {
   return {b, total, gridDim.x};
 }
 
-template <class L, int MAXE, bool ZERO>
+template <class L, int MAXE, bool ZERO, bool MIS>
 __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
     commit_kernel(const __grid_constant__ CommitPlan<MAXE> plan, unsigned long long *out) {
+  constexpr uint32_t kPad = MIS ? 16 : 0, kStage = stage_bytes<L, MIS>();
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(8) uint64_t full[L::kStages];
   __shared__ __align__(8) uint64_t empty[L::kStages];
@@ -370,44 +495,69 @@ __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
   Acc a{0, 0, 0, 0};
   if (warp == L::kConsumerWarps) {
     // ------------------------------------------------------------ producer
+    const Scalars s{plan.h, plan.one};
+    uint32_t phase = 0;
+    int stage = 0;
+    uint64_t issued = 0;
     if (lane == 0) {
       const uint64_t policy = l2_evict_first();
-      uint32_t cur = 0, phase = 0;
-      int stage = 0;
-      uint64_t issued = 0;
+      uint32_t cur = 0;
       const TileWalk w = tile_walk(plan.total_tiles);
       for (uint64_t tile = w.t0; tile < w.t1; tile += w.ts) {
         if (*(volatile int *)&abort_flag) break;
         cur = find_tile(plan, cur, tile);
         const CommitEntry &E = plan.e[cur];
         const uint64_t start = E.head + (tile - E.tile_begin) * L::kTile;
-        const uint64_t vec_end = E.head + ((E.n - E.head) & ~(uint64_t)7);
-        const uint32_t cnt = (uint32_t)umin64(L::kTile, vec_end - start);
+        const uint32_t cnt = (uint32_t)umin64(L::kTile, E.head + E.body - start);
         if (!mbar_wait(&empty[stage], phase ^ 1)) {
           fail_wait(&abort_flag);
           break;
         }
-        uint8_t *st = smem + (size_t)stage * stage_bytes<L>();
-        desc[stage] = StageDesc{static_cast<uint8_t *>(E.p) + start * L::kES,
-                                static_cast<uint8_t *>(E.m) + start * L::kES,
-                                static_cast<uint8_t *>(E.v) + start * L::kES,
-                                L::kDigests == 4 ? E.w + start : nullptr,
-                                const_cast<uint16_t *>(E.g) + start,
-                                cnt,
-                                E.key_base + (uint32_t)start};
-        mbar_arrive_expect_tx(&full[stage], cnt * (3 * L::kES + 2));
-        bulk_g2s(st, static_cast<const uint8_t *>(E.p) + start * L::kES, cnt * L::kES, &full[stage], policy);
-        bulk_g2s(st + L::kES * L::kTile, static_cast<const uint8_t *>(E.m) + start * L::kES, cnt * L::kES,
-                 &full[stage], policy);
-        bulk_g2s(st + 2 * L::kES * L::kTile, static_cast<const uint8_t *>(E.v) + start * L::kES,
-                 cnt * L::kES, &full[stage], policy);
-        bulk_g2s(st + 3 * L::kES * L::kTile, E.g + start, cnt * 2, &full[stage], policy);
+        uint8_t *st = smem + (size_t)stage * kStage;
+        uint8_t *const p = static_cast<uint8_t *>(E.p) + start * L::kES, *const m = static_cast<uint8_t *>(E.m) + start * L::kES,
+                *const v = static_cast<uint8_t *>(E.v) + start * L::kES;
+        uint16_t *const g = const_cast<uint16_t *>(E.g) + start;
+        constexpr uint32_t kRegion = L::kES * (uint32_t)L::kTile + kPad;
+        StageDesc sd{p, m, v, L::kDigests == 4 ? E.w + start : nullptr, g, cnt, E.key_base + (uint32_t)start};
+        if (MIS && E.mis) {
+          const auto off = [](const void *x) { return (uint32_t)((uintptr_t)x & 15); };
+          const auto blocks = [&](const void *x, uint32_t bytes) { return (off(x) + bytes + 15) & ~15u; };
+          sd.cnt |= kMisTile | off(p) << 16 | off(m) << 20 | off(v) << 24 | off(g) << 28;
+          desc[stage] = sd;
+          mbar_arrive_expect_tx(&full[stage], blocks(p, cnt * L::kES) + blocks(m, cnt * L::kES) +
+                                                  blocks(v, cnt * L::kES) + blocks(g, cnt * 2));
+          copy_blocks(st, p, cnt * L::kES, &full[stage], policy);
+          copy_blocks(st + kRegion, m, cnt * L::kES, &full[stage], policy);
+          copy_blocks(st + 2 * kRegion, v, cnt * L::kES, &full[stage], policy);
+          copy_blocks(st + 3 * kRegion, reinterpret_cast<const uint8_t *>(g), cnt * 2, &full[stage], policy);
+        } else {
+          desc[stage] = sd;
+          mbar_arrive_expect_tx(&full[stage], cnt * (3 * L::kES + 2));
+          bulk_g2s(st, p, cnt * L::kES, &full[stage], policy);
+          bulk_g2s(st + kRegion, m, cnt * L::kES, &full[stage], policy);
+          bulk_g2s(st + 2 * kRegion, v, cnt * L::kES, &full[stage], policy);
+          bulk_g2s(st + 3 * kRegion, g, cnt * 2, &full[stage], policy);
+        }
         ++issued;
         if (++stage == L::kStages) {
           stage = 0;
           phase ^= 1;
         }
       }
+    }
+    __syncwarp();
+    // With its copies issued, the producer warp does what the entries hold
+    // outside their tiles, one entry at a time: up to 8 elements before
+    // (lanes 0-7) and 24 behind (lanes 8-31).
+    for (uint32_t e = blockIdx.x; e < plan.count; e += gridDim.x) {
+      const CommitEntry &E = plan.e[e];
+      const uint64_t i = lane < 8 ? lane : E.head + E.body + (lane - 8);
+      if (i < (lane < 8 ? (uint64_t)E.head : E.n)) {
+        L::one(E, i, s, a);
+        if (ZERO) const_cast<uint16_t *>(E.g)[i] = 0;
+      }
+    }
+    if (lane == 0) {
       // Drain: the last min(issued, stages) copies must have landed before
       // the CTA may exit (normally the consumers already waited for them).
       const int n_drain = (int)umin64(issued, (uint64_t)L::kStages);
@@ -434,44 +584,36 @@ __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
       }
       if (*(volatile int *)&abort_flag) break;
       const StageDesc sd = desc[stage];
-      const uint8_t *st = smem + (size_t)stage * stage_bytes<L>();
-      typename L::Regs r[L::kGroups];
-      bool ok[L::kGroups];
+      const uint8_t *st = smem + (size_t)stage * kStage;
+      if (MIS && (sd.cnt & kMisTile)) {
+        const uint32_t cnt = sd.cnt & (kMisTile - 1);
+        const typename L::Mis x(st, sd.cnt);
+        uint32_t e = ct;
+#pragma unroll L::kMisUnroll
+        for (; e + L::kConsumers < cnt; e += 2 * L::kConsumers) L::template mis_pair<ZERO>(sd, x, e, s, a);
+        if (e < cnt) L::template mis_one<ZERO>(sd, x, e, s, a);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[stage]);
+      } else {
+        typename L::Regs r[L::kGroups];
+        bool ok[L::kGroups];
 #pragma unroll
-      for (int k = 0; k < L::kGroups; ++k) {
-        const uint32_t e = (uint32_t)(k * L::kConsumers + ct) * 4;
-        ok[k] = e < sd.cnt;
-        if (ok[k]) L::load(st, e, r[k]);
+        for (int k = 0; k < L::kGroups; ++k) {
+          const uint32_t e = (uint32_t)(k * L::kConsumers + ct) * 4;
+          ok[k] = e < sd.cnt;
+          if (ok[k]) L::template load<kPad>(st, e, r[k]);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[stage]);
+        // this thread's first element in the tile is element 4 * ct
+        const uint32_t ob = 4u * (uint32_t)ct;
+        const Dst d{sd.p + ob * L::kES, sd.m + ob * L::kES, sd.v + ob * L::kES,
+                    L::kDigests == 4 ? sd.w + ob : nullptr, sd.g + ob};
+        store_groups<L, ZERO, 0>(d, sd.G + ob, r, ok, s, a);
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&empty[stage]);
-      // this thread's first element in the tile is element 4 * ct
-      const uint32_t ob = 4u * (uint32_t)ct;
-      const Dst d{sd.p + ob * L::kES, sd.m + ob * L::kES, sd.v + ob * L::kES,
-                  L::kDigests == 4 ? sd.w + ob : nullptr, sd.g + ob};
-      store_groups<L, ZERO, 0>(d, sd.G + ob, r, ok, s, a);
       if (++stage == L::kStages) {
         stage = 0;
         phase ^= 1;
-      }
-    }
-    // scalar items: entry heads and tails, and entries without vectors
-    if (!*(volatile int *)&abort_flag) {
-      uint32_t cur = 0;
-      for (uint64_t it = (uint64_t)blockIdx.x * L::kConsumers + ct; it < plan.total_scalar;
-           it += (uint64_t)gridDim.x * L::kConsumers) {
-        while (cur + 1 < plan.count && it >= plan.e[cur + 1].scalar_begin) ++cur;
-        const CommitEntry &E = plan.e[cur];
-        const uint64_t k = it - E.scalar_begin;
-        uint64_t i;
-        if (E.head == kScalarMode) {
-          i = k;
-        } else {
-          const uint64_t vec_end = E.head + ((E.n - E.head) & ~(uint64_t)7);
-          i = k < E.head ? k : vec_end + (k - E.head);
-        }
-        L::one(E, i, s, a);
-        if (ZERO) const_cast<uint16_t *>(E.g)[i] = 0;
       }
     }
   }
@@ -502,7 +644,7 @@ __global__ void wait_timeout_kernel(uint64_t limit_ns) {
 // The dynamic shared-memory limit of one kernel instantiation, raised once
 // per device (the first launch on a device sets it; later launches, for
 // example inside a stream capture, only enqueue).
-template <class L, int MAXE, bool ZERO>
+template <class L, int MAXE, bool ZERO, bool MIS>
 int ensure_smem_attribute() {
   static std::atomic<uint64_t> done_mask{0};
   int dev = 0;
@@ -510,11 +652,11 @@ int ensure_smem_attribute() {
   if (e != cudaSuccess) return (int)e;
   const uint64_t bit = dev < 64 ? (1ull << dev) : 0;
   if (bit && (done_mask.load(std::memory_order_acquire) & bit)) return 0;
-  e = cudaFuncSetAttribute(commit_kernel<L, MAXE, ZERO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem_bytes<L>());
+  e = cudaFuncSetAttribute(commit_kernel<L, MAXE, ZERO, MIS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)smem_bytes<L, MIS>());
   if (e != cudaSuccess) return (int)e;
   if (APC_SMEM_CARVEOUT >= 0) {
-    e = cudaFuncSetAttribute(commit_kernel<L, MAXE, ZERO>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    e = cudaFuncSetAttribute(commit_kernel<L, MAXE, ZERO, MIS>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              APC_SMEM_CARVEOUT);
     if (e != cudaSuccess) return (int)e;
   }
@@ -522,30 +664,48 @@ int ensure_smem_attribute() {
   return 0;
 }
 
-template <class L, int MAXE, bool ZERO>
+template <class L, int MAXE, bool ZERO, bool MIS>
 int launch_t(const CommitPlan<MAXE> &plan, unsigned grid, void *stream, unsigned long long *out) {
-  int e = ensure_smem_attribute<L, MAXE, ZERO>();
+  int e = ensure_smem_attribute<L, MAXE, ZERO, MIS>();
   if (e) return e;
-  commit_kernel<L, MAXE, ZERO><<<grid, L::kThreads, smem_bytes<L>(), (cudaStream_t)stream>>>(plan, out);
+  commit_kernel<L, MAXE, ZERO, MIS>
+      <<<grid, L::kThreads, smem_bytes<L, MIS>(), (cudaStream_t)stream>>>(plan, out);
   return (int)cudaGetLastError();
+}
+
+template <class L, int MAXE>
+int launch_l(const CommitPlan<MAXE> &plan, bool zero_grad, unsigned grid, void *stream, unsigned long long *out) {
+  bool mis = false;
+  for (uint32_t k = 0; k < plan.count; ++k) mis |= plan.e[k].mis != 0;
+  if (mis)
+    return zero_grad ? launch_t<L, MAXE, true, true>(plan, grid, stream, out)
+                     : launch_t<L, MAXE, false, true>(plan, grid, stream, out);
+  return zero_grad ? launch_t<L, MAXE, true, false>(plan, grid, stream, out)
+                   : launch_t<L, MAXE, false, false>(plan, grid, stream, out);
 }
 
 template <int MAXE>
 int launch(const CommitPlan<MAXE> &plan, int layout, bool zero_grad, unsigned grid, void *stream,
            unsigned long long *out) {
-  if (layout == kLayoutBF16)
-    return zero_grad ? launch_t<BF16State, MAXE, true>(plan, grid, stream, out)
-                     : launch_t<BF16State, MAXE, false>(plan, grid, stream, out);
-  return zero_grad ? launch_t<F32State, MAXE, true>(plan, grid, stream, out)
-                   : launch_t<F32State, MAXE, false>(plan, grid, stream, out);
+  return layout == kLayoutBF16 ? launch_l<BF16State>(plan, zero_grad, grid, stream, out)
+                               : launch_l<F32State>(plan, zero_grad, grid, stream, out);
+}
+
+template <class L, int MAXE, bool MIS>
+int blocks_m(int *out) {
+  int e = ensure_smem_attribute<L, MAXE, false, MIS>();
+  if (e) return e;
+  return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, commit_kernel<L, MAXE, false, MIS>, L::kThreads,
+                                                            smem_bytes<L, MIS>());
 }
 
 template <class L, int MAXE>
 int blocks_per_sm(int *out) {
-  int e = ensure_smem_attribute<L, MAXE, false>();
-  if (e) return e;
-  return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, commit_kernel<L, MAXE, false>, L::kThreads,
-                                                            smem_bytes<L>());
+  int a = 0, b = 0;
+  int e = blocks_m<L, MAXE, false>(&a);
+  if (e || (e = blocks_m<L, MAXE, true>(&b))) return e;
+  *out = a < b ? a : b;
+  return 0;
 }
 
 }  // namespace
@@ -561,7 +721,7 @@ int launch_commit_large(const CommitPlan<kCommitLarge> &plan, int layout, bool z
 }
 
 int commit_blocks_per_sm(bool large, int *out) {
-  // one grid size serves both layouts: the smaller of their residencies
+  // one grid size serves all instantiations: the smaller of their residencies
   int f = 0, b = 0;
   int e = large ? blocks_per_sm<F32State, kCommitLarge>(&f) : blocks_per_sm<F32State, kCommitSmall>(&f);
   if (e) return e;

@@ -187,8 +187,8 @@ apc_status check_device_pointers(std::vector<Owned> &ptrs) {
   return APC_OK;
 }
 
-// Entries arrive with their tile count in tile_begin and their scalar-item
-// count in scalar_begin; each batch turns both into prefix offsets.
+// Entries arrive with their tile count in tile_begin; each batch turns it into
+// prefix offsets.
 template <int MAXE, typename Launch>
 apc_status run_commit_batches(const std::vector<apc::CommitEntry> &entries, const float h[8], int layout,
                               bool zero_grad, unsigned grid_cap, void *stream, unsigned long long *out,
@@ -199,21 +199,17 @@ apc_status run_commit_batches(const std::vector<apc::CommitEntry> &entries, cons
   size_t i = 0;
   while (i < entries.size()) {
     const size_t k = std::min(entries.size() - i, (size_t)MAXE);
-    uint64_t tiles = 0, scalars = 0;
+    uint64_t tiles = 0;
     for (size_t j = 0; j < k; ++j) {
       apc::CommitEntry e = entries[i + j];
-      const uint64_t t = e.tile_begin, sc = e.scalar_begin;
+      const uint64_t t = e.tile_begin;
       e.tile_begin = tiles;
-      e.scalar_begin = scalars;
       tiles += t;
-      scalars += sc;
       plan->e[j] = e;
     }
     plan->count = (uint32_t)k;
     plan->total_tiles = tiles;
-    plan->total_scalar = scalars;
-    const uint64_t consumers = (uint64_t)apc::commit_consumers(layout);
-    const uint64_t want = std::max<uint64_t>(tiles, (scalars + consumers - 1) / consumers);
+    const uint64_t want = std::max<uint64_t>(tiles, k);
     const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(want, grid_cap));
     int e = launch(*plan, layout, zero_grad, grid, stream, out);
     if (e) return cuda_fail(e, "commit kernel launch");
@@ -326,17 +322,14 @@ apc_status commit_common(int layout, const std::vector<TableRow> &rows, const ap
     e.w = t.w;
     e.n = t.n;
     e.key_base = (uint32_t)t.goff;
-    if (aligned) {
-      const uint64_t head = std::min<uint64_t>(h0, t.n);
-      const uint64_t body = (t.n - head) / apc::kVec * apc::kVec;
-      e.head = (uint32_t)head;
-      e.tile_begin = ceil_div(body, apc::commit_tile(layout));  // tile count until placed
-      e.scalar_begin = t.n - body;                       // head + tail items
-    } else {
-      e.head = apc::kScalarMode;
-      e.tile_begin = 0;
-      e.scalar_begin = t.n;
-    }
+    // aligned: whole 16-byte vectors from there on; misaligned: 8 elements left
+    // out on either side, all of them where that leaves no vector
+    const uint64_t head = std::min<uint64_t>(aligned ? h0 : 8, t.n);
+    const uint64_t room = t.n - head - (aligned ? 0 : std::min<uint64_t>(8, t.n - head));
+    e.head = (uint16_t)head;
+    e.body = t.n < 32 && !aligned ? 0 : room / apc::kVec * apc::kVec;
+    e.mis = !aligned && e.body;
+    e.tile_begin = ceil_div(e.body, apc::commit_tile(layout));  // tile count until placed
     entries.push_back(e);
   }
   const uintptr_t o = (uintptr_t)out_digests;

@@ -11,7 +11,6 @@
 namespace apc {
 
 constexpr int kVec = 8;                    // vector granularity: 16 bytes of bf16, 32 bytes of fp32
-constexpr uint32_t kScalarMode = 0xFFFFFFFFu;  // `head` value of an entry run without vectors
 
 // Commit kernel: warp-specialized pipeline.  One producer warp streams each
 // tile of p, m, v and g into a ring of shared-memory stages with bulk
@@ -96,36 +95,33 @@ constexpr int kLayoutF32 = 0;   // fp32 p, m, v; bf16 g; bf16 copy w
 constexpr int kLayoutBF16 = 1;  // bf16 p, m, v; bf16 g; no copy
 
 constexpr uint64_t commit_tile(int layout) { return layout == kLayoutBF16 ? kCommitTileBF16 : kCommitTile; }
-constexpr int commit_consumers(int layout) {
-  return 32 * (layout == kLayoutBF16 ? kCommitConsumerWarpsBF16 : kCommitConsumerWarps);
-}
 
 // One chunk-table entry of the commit kernel (72 bytes).
 //   p, m, v: fp32 or bf16 state (by the launch's layout); w: the bf16 copy
 //         (fp32 layout only).
-//   head: elements [0, head) are scalar items, then 16-byte aligned vectors
-//         up to vec_end = head + 8 * floor((n - head) / 8) in tiles of
-//         commit_tile(layout), then scalar items up to n; kScalarMode when the
-//         buffers are not mutually 16-byte aligned (all n elements scalar).
+//   head, body: elements [head, head + body) run in tiles of
+//         commit_tile(layout), the up to 8 before and 24 behind one by one.
+//   mis:  the buffers are not mutually 16-byte aligned.  Then the blocks of 16
+//         bytes that hold the body reach at most 15 bytes over it, which
+//         stays inside the buffers (8 elements are left out on either side).
 //   tile_begin: the entry's first tile in the launch's tile space.
-//   scalar_begin: the entry's first item in the launch's scalar-item space.
 //   key_base: global_offset mod 2^32 (the digest key of element 0).
 struct CommitEntry {
   void *p, *m, *v;
   const uint16_t *g;
   uint16_t *w;
   uint64_t n;
+  uint64_t body;
   uint64_t tile_begin;
-  uint64_t scalar_begin;
   uint32_t key_base;
-  uint32_t head;
+  uint16_t head;
+  uint16_t mis;
 };
 
 template <int MAXE>
 struct CommitPlan {
   float h[8];            // b1, 1-b1, b2, 1-b2, eps, 1-lr*wd, lr/bc1, 1/sqrt(bc2)
   uint64_t total_tiles;
-  uint64_t total_scalar;
   uint32_t count;
   uint32_t one;          // 1: the FMA-pipe carry-add multiplier of the digest
   CommitEntry e[MAXE];

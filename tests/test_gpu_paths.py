@@ -6,6 +6,7 @@ import pytest
 import torch
 
 import oracle
+import synth
 import paper_2609_18178_gb300 as apc
 from apc_testlib import M64
 
@@ -97,3 +98,90 @@ def test_digest_many_short_buffers():
         bufs.append(apc.BufferEntry(d[at:at + n], slot, goff, apc.F32 if f32 else apc.BF16))
         at += n
     assert apc.digests_to_host(apc.digest(bufs, 5)) == want
+
+
+def committed(tensors, offs, step, layout, zero, shifts):
+    """Commit `tensors` (dicts p, m, v, g of numpy words, goff), each buffer
+    placed `shifts[buffer]` elements into its allocation; (results, digests)
+    of the device and of the oracle."""
+    f32 = layout == "f32"
+    hp = oracle.DEFAULT_HP
+    entries, devs = [], []
+    for i, t in enumerate(tensors):
+        d = {}
+        for k in ("p", "m", "v", "g") + (("w",) if f32 else ()):
+            a = t[k] if k != "w" else np.zeros(t["g"].size, np.uint16)
+            s = shifts[(i, k)]
+            buf = torch.zeros(a.size + 40, dtype=torch.int32 if a.itemsize == 4 else torch.int16, device="cuda")
+            buf.fill_(0x55)
+            buf[s:s + a.size] = torch.from_numpy(a.view(np.int32 if a.itemsize == 4 else np.int16).copy()).cuda()
+            d[k] = (buf, s, a.size)
+        devs.append(d)
+        v = {k: b[s:s + n] for k, (b, s, n) in d.items()}
+        entries.append(apc.TensorEntry(v["p"], v["m"], v["v"], v["g"], v["w"], offs[i]) if f32 else
+                       apc.TensorEntryBF16(v["p"], v["m"], v["v"], v["g"], offs[i]))
+    out = (apc.commit_step if f32 else apc.commit_step_bf16)(entries, step, hp, zero_grad=zero)
+    torch.cuda.synchronize()
+    h8 = oracle.resolve_hparams(hp, step)
+    want = [0] * (4 if f32 else 3)
+    for t, d, off in zip(tensors, devs, offs):
+        ref = {k: t[k].copy() for k in "pmv"}
+        if f32:
+            ref = {k: a.view(np.float32) for k, a in ref.items()}
+            ref["w"], dg = oracle.commit(ref["p"], ref["m"], ref["v"], t["g"], off, h8)
+        else:
+            dg = oracle.commit_bf16(ref["p"], ref["m"], ref["v"], t["g"], off, h8)
+        want = [(a + b) & M64 for a, b in zip(want, dg)]
+        ref["g"] = np.zeros_like(t["g"]) if zero else t["g"]
+        for k, (buf, s, n) in d.items():
+            got = buf.cpu().numpy()
+            r = ref[k].view(got.dtype)
+            assert np.array_equal(got[s:s + n], r), (k, n, s)
+            assert (got[:s] == 0x55).all() and (got[s + n:] == 0x55).all(), (k, n, s, "outside the buffer")
+    assert apc.digests_to_host(out) == want
+
+
+def state_words(n, goff, step, layout):
+    if layout == "f32":
+        p, m, v = synth.state(n, goff)
+        return dict(p=p.view(np.uint32), m=m.view(np.uint32), v=v.view(np.uint32), g=synth.grad(n, goff, step))
+    p, m, v = synth.state_bf16(n, goff)
+    return dict(p=p, m=m, v=v, g=synth.grad(n, goff, step))
+
+
+# Elements per tile of the commit kernel and the sizes around its edges; a
+# misaligned entry runs 8 elements on either side and entries under 32 apart.
+TILE = {"f32": 4864, "bf16": 10368}
+
+
+@pytest.mark.parametrize("zero", [False, True])
+@pytest.mark.parametrize("layout", ["f32", "bf16"])
+def test_commit_misaligned_entries(layout, zero):
+    """Entries whose buffers sit at different offsets from a 16-byte boundary,
+    of every size near the path's edges, mixed with aligned ones; nothing
+    outside a buffer changes."""
+    rng = np.random.default_rng(21)
+    t = TILE[layout]
+    sizes = list(range(1, 12)) + [15, 16, 23, 24, 25, 31, 32, 33, 39, 40, 41, 1000, t - 1, t, t + 1, t + 15, t + 16, t + 17,
+                                  t + 24, t + 25, 2 * t + 16, 2 * t + 40, 3 * t - 7]
+    tensors, offs, shifts = [], [], {}
+    for i, n in enumerate(sizes):
+        goff = int(rng.integers(0, 1 << 33))
+        tensors.append(state_words(n, goff, 4, layout))
+        offs.append(goff)
+        same = int(rng.integers(0, 16))
+        for k in "pmvgw":
+            shifts[(i, k)] = same if i % 5 == 4 else int(rng.integers(0, 16))
+    committed(tensors, offs, 4, layout, zero, shifts)
+
+
+@pytest.mark.parametrize("layout", ["f32", "bf16"])
+def test_commit_every_relative_offset(layout):
+    """One tile's worth of elements at every offset of the gradient (and copy)
+    against the state, each in a launch of its own."""
+    n = TILE[layout] + 77
+    t = state_words(n, 12345, 9, layout)
+    for gs in range(8):
+        for ps in range(0, 4 if layout == "f32" else 8):
+            committed([t], [12345], 9, layout, False,
+                      {(0, "p"): ps, (0, "m"): (ps + gs) % 8, (0, "v"): 3, (0, "g"): gs, (0, "w"): (gs + 1) % 8})
