@@ -13,8 +13,9 @@
 //
 // Warp-specialized pipeline (one persistent CTA per SM by default):
 //  * The producer warp walks the CTA's run of the launch's tiles (one
-//    contiguous run per CTA; a tile is L::kTile elements of one entry's
-//    16-byte aligned body: 4,864 for fp32 state, 10,368 for bf16 state)
+//    contiguous run per CTA; a tile is up to L::kTile elements of one entry's
+//    16-byte aligned body: 4,864 for fp32 state, 10,368 for bf16 state; less
+//    in small launches, where the host chooses plan.tile for balance)
 //    and, for each, waits until a ring stage is free and issues four
 //    bulk asynchronous copies -- p, m, v and g -- that complete on the
 //    stage's "full" mbarrier.  Loads never occupy consumer registers, and up
@@ -449,6 +450,21 @@ __device__ __forceinline__ void copy_blocks(uint8_t *dst, const uint8_t *src, ui
   bulk_g2s(dst, src - off, (off + bytes + 15) & ~15u, bar, policy);
 }
 
+// The entry that holds `tile` (the last that begins at or before it; entries
+// without tiles begin where the next one does), by bisection: a walk from the
+// first entry took 440 dependent constant loads in a CTA near a full table's
+// end.  The producer then walks on from there.
+template <int MAXE>
+__device__ __forceinline__ uint32_t first_entry(const CommitPlan<MAXE> &plan, uint64_t tile) {
+  uint32_t lo = 0, hi = plan.count;
+  while (hi - lo > 1) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (plan.e[mid].tile_begin <= tile) lo = mid;
+    else hi = mid;
+  }
+  return lo;
+}
+
 template <int MAXE>
 __device__ __forceinline__ uint32_t find_tile(const CommitPlan<MAXE> &plan, uint32_t cur, uint64_t tile) {
   while (cur + 1 < plan.count && tile >= plan.e[cur + 1].tile_begin) ++cur;
@@ -478,7 +494,7 @@ __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
   __shared__ __align__(8) uint64_t full[L::kStages];
   __shared__ __align__(8) uint64_t empty[L::kStages];
   __shared__ StageDesc desc[L::kStages];
-  __shared__ uint64_t red[L::kThreads / 32];
+  __shared__ uint64_t red[L::kDigests][L::kThreads / 32];
   __shared__ int abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -501,14 +517,14 @@ __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
     uint64_t issued = 0;
     if (lane == 0) {
       const uint64_t policy = l2_evict_first();
-      uint32_t cur = 0;
       const TileWalk w = tile_walk(plan.total_tiles);
+      uint32_t cur = w.t0 < w.t1 ? first_entry(plan, w.t0) : 0;
       for (uint64_t tile = w.t0; tile < w.t1; tile += w.ts) {
         if (*(volatile int *)&abort_flag) break;
         cur = find_tile(plan, cur, tile);
         const CommitEntry &E = plan.e[cur];
-        const uint64_t start = E.head + (tile - E.tile_begin) * L::kTile;
-        const uint32_t cnt = (uint32_t)umin64(L::kTile, E.head + E.body - start);
+        const uint64_t start = E.head + (tile - E.tile_begin) * plan.tile;
+        const uint32_t cnt = (uint32_t)umin64(plan.tile, E.head + E.body - start);
         if (!mbar_wait(&empty[stage], phase ^ 1)) {
           fail_wait(&abort_flag);
           break;
@@ -618,17 +634,16 @@ __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
     }
   }
 
-  const bool ok = !*(volatile int *)&abort_flag;
-  uint64_t r;
-  r = cta_sum<L::kThreads>(a.p, red);
-  if (threadIdx.x == 0 && ok && r) atomicAdd(&out[0], (unsigned long long)r);
-  r = cta_sum<L::kThreads>(a.m, red);
-  if (threadIdx.x == 0 && ok && r) atomicAdd(&out[1], (unsigned long long)r);
-  r = cta_sum<L::kThreads>(a.v, red);
-  if (threadIdx.x == 0 && ok && r) atomicAdd(&out[2], (unsigned long long)r);
-  if (L::kDigests == 4) {
-    r = cta_sum<L::kThreads>(a.w, red);
-    if (threadIdx.x == 0 && ok && r) atomicAdd(&out[3], (unsigned long long)r);
+  // each warp sums its lanes' digests; after one barrier warp d adds the
+  // warps' sums of digest d into the output
+  const uint64_t sums[4] = {warp_sum(a.p), warp_sum(a.m), warp_sum(a.v), L::kDigests == 4 ? warp_sum(a.w) : 0};
+  if (lane == 0)
+#pragma unroll
+    for (int d = 0; d < L::kDigests; ++d) red[d][warp] = sums[d];
+  __syncthreads();
+  if (warp < L::kDigests && !*(volatile int *)&abort_flag) {
+    const uint64_t r = warp_sum(lane < L::kThreads / 32 ? red[warp][lane] : 0);
+    if (lane == 0 && r) atomicAdd(&out[warp], (unsigned long long)r);
   }
 }
 

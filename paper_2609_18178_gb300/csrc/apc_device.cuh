@@ -261,22 +261,11 @@ __device__ __forceinline__ void acc_add(uint64_t &acc, uint64_t z, uint32_t one)
   acc = ((uint64_t)ahi << 32) | alo;
 }
 
-// Sum of a CTA's per-thread values; the result is valid in thread 0.
-// `scratch` holds THREADS/32 words.
-template <int THREADS>
-__device__ __forceinline__ uint64_t cta_sum(uint64_t x, uint64_t *scratch) {
+// Sum of a warp's values, in every lane.
+__device__ __forceinline__ uint64_t warp_sum(uint64_t x) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) scratch[warp] = x;
-  __syncthreads();
-  uint64_t r = 0;
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int i = 0; i < THREADS / 32; ++i) r += scratch[i];
-  }
-  __syncthreads();
-  return r;
+  return x;
 }
 
 }  // namespace apc

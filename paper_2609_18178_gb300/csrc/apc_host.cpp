@@ -65,6 +65,8 @@ apc_status resolve(const apc_adamw_hparams *hp, int64_t step, float out[8]) {
   return APC_OK;
 }
 
+uint64_t ceil_div(uint64_t a, uint64_t b) { return a / b + (a % b != 0); }
+
 struct Range {
   uintptr_t lo, hi;  // [lo, hi)
   bool written;
@@ -187,8 +189,43 @@ apc_status check_device_pointers(std::vector<Owned> &ptrs) {
   return APC_OK;
 }
 
-// Entries arrive with their tile count in tile_begin; each batch turns it into
-// prefix offsets.
+// Elements per tile of one launch.  The full tile is what the ring is built
+// for, and the launch's time is then set by bandwidth.  In a launch of few
+// rounds of them it is set by the CTA with the most to do: 1 M elements are
+// 216 full tiles for 152 CTAs, two rounds for 64 of them and one for the rest,
+// and 100,000 elements are 21 tiles for 21 CTAs.  So up to kEvenRounds rounds
+// the length is chosen that gives that CTA the least work, a tile counting as
+// its elements and kTileCost more (its share of the pipeline's latency; 256
+// and 1,024 measure the same).  With the kernel's bisection and its one-barrier
+// sum, 100,003 elements take 5.5 us of kernel time (9.1 before), 1 M take 11.4
+// (13.3), 1,100 entries of 136 to 20,557 take 50 in three launches (130).
+constexpr uint64_t kEvenRounds = 8, kTileCost = 512, kTileStep = 64, kTileMin = 256;
+
+uint32_t commit_launch_tile(const apc::CommitEntry *e, size_t count, uint64_t full, uint64_t grid) {
+  uint64_t body = 0, longest = 0;
+  for (size_t j = 0; j < count; ++j) {
+    body += e[j].body;
+    longest = std::max(longest, e[j].body);
+  }
+  if (body > kEvenRounds * grid * full) return (uint32_t)full;
+  uint64_t best = full, best_cost = UINT64_MAX;
+  const uint64_t fewest = std::max<uint64_t>(1, ceil_div(body, grid * full));
+  for (uint64_t rounds = fewest; rounds < fewest + 4; ++rounds) {
+    const uint64_t even = ceil_div(ceil_div(body, grid * rounds), kTileStep) * kTileStep;
+    const uint64_t tile = std::min(full, std::max(kTileMin, even));
+    const double per = 1.0 / (double)tile;  // an estimate will do here
+    uint64_t tiles = 0;
+    for (size_t j = 0; j < count; ++j) tiles += (uint64_t)((double)(e[j].body + tile - 1) * per);
+    const uint64_t cost = ceil_div(tiles, grid) * (std::min(tile, longest) + kTileCost);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = tile;
+    }
+  }
+  return (uint32_t)best;
+}
+
+// Entries arrive without tile_begin; each batch places their tiles.
 template <int MAXE, typename Launch>
 apc_status run_commit_batches(const std::vector<apc::CommitEntry> &entries, const float h[8], int layout,
                               bool zero_grad, unsigned grid_cap, void *stream, unsigned long long *out,
@@ -199,14 +236,15 @@ apc_status run_commit_batches(const std::vector<apc::CommitEntry> &entries, cons
   size_t i = 0;
   while (i < entries.size()) {
     const size_t k = std::min(entries.size() - i, (size_t)MAXE);
+    const uint32_t tile = commit_launch_tile(&entries[i], k, apc::commit_tile(layout), grid_cap);
     uint64_t tiles = 0;
     for (size_t j = 0; j < k; ++j) {
       apc::CommitEntry e = entries[i + j];
-      const uint64_t t = e.tile_begin;
       e.tile_begin = tiles;
-      tiles += t;
+      tiles += ceil_div(e.body, tile);
       plan->e[j] = e;
     }
+    plan->tile = tile;
     plan->count = (uint32_t)k;
     plan->total_tiles = tiles;
     const uint64_t want = std::max<uint64_t>(tiles, k);
@@ -247,8 +285,6 @@ apc_status run_digest_batches(const std::vector<apc::DigestEntry> &entries, unsi
   }
   return APC_OK;
 }
-
-uint64_t ceil_div(uint64_t a, uint64_t b) { return a / b + (a % b != 0); }
 
 }  // namespace
 
@@ -329,7 +365,6 @@ apc_status commit_common(int layout, const std::vector<TableRow> &rows, const ap
     e.head = (uint16_t)head;
     e.body = t.n < 32 && !aligned ? 0 : room / apc::kVec * apc::kVec;
     e.mis = !aligned && e.body;
-    e.tile_begin = ceil_div(e.body, apc::commit_tile(layout));  // tile count until placed
     entries.push_back(e);
   }
   const uintptr_t o = (uintptr_t)out_digests;

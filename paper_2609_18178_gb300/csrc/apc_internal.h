@@ -99,8 +99,8 @@ constexpr uint64_t commit_tile(int layout) { return layout == kLayoutBF16 ? kCom
 // One chunk-table entry of the commit kernel (72 bytes).
 //   p, m, v: fp32 or bf16 state (by the launch's layout); w: the bf16 copy
 //         (fp32 layout only).
-//   head, body: elements [head, head + body) run in tiles of
-//         commit_tile(layout), the up to 8 before and 24 behind one by one.
+//   head, body: elements [head, head + body) run in tiles of the plan's `tile`
+//         elements, the up to 8 before and 24 behind one by one.
 //   mis:  the buffers are not mutually 16-byte aligned.  Then the blocks of 16
 //         bytes that hold the body reach at most 15 bytes over it, which
 //         stays inside the buffers (8 elements are left out on either side).
@@ -124,6 +124,8 @@ struct CommitPlan {
   uint64_t total_tiles;
   uint32_t count;
   uint32_t one;          // 1: the FMA-pipe carry-add multiplier of the digest
+  uint32_t tile;         // elements per tile of this launch (a multiple of 64, at most commit_tile)
+  uint32_t pad_;
   CommitEntry e[MAXE];
 };
 

@@ -185,3 +185,19 @@ def test_commit_every_relative_offset(layout):
         for ps in range(0, 4 if layout == "f32" else 8):
             committed([t], [12345], 9, layout, False,
                       {(0, "p"): ps, (0, "m"): (ps + gs) % 8, (0, "v"): 3, (0, "g"): gs, (0, "w"): (gs + 1) % 8})
+
+
+@pytest.mark.parametrize("layout", ["f32", "bf16"])
+@pytest.mark.parametrize("limit", [1, 3])
+def test_commit_launch_tiles(monkeypatch, layout, limit):
+    """Launches on either side of the lengths where the tile changes: the
+    shortest tile, even shares of one to several rounds, and the full tile
+    from more than eight rounds on; alone and beside short entries."""
+    grid_limit(monkeypatch, limit)
+    t = TILE[layout] * limit
+    for n in (255, 256, 257, 256 * limit + 8, t - 8, t, t + 8, 2 * t + 1, 5 * t + 64, 8 * t - 8, 8 * t, 8 * t + 8, 8 * t + 9):
+        tensors = [state_words(m, 77, 2, layout) for m in (n, 33, 5, 700)]
+        shifts = {(i, k): 0 for i in range(4) for k in "pmvgw"}
+        shifts[(1, "g")] = 1
+        committed(tensors[:1], [77], 2, layout, False, shifts)
+        committed(tensors, [77] * 4, 2, layout, True, shifts)
