@@ -125,7 +125,7 @@ def _check(status: int) -> None:
 
 
 def _hp(hp: dict | None) -> _HParams:
-    hp = dict(DEFAULT_HPARAMS, **(hp or {}))
+    hp = dict(DEFAULT_HPARAMS, **hp) if hp else DEFAULT_HPARAMS
     return _HParams(hp["lr"], hp["beta1"], hp["beta2"], hp["eps"], hp["weight_decay"])
 
 
@@ -155,7 +155,8 @@ def _ptr(x, itemsize: int | None = None) -> int:
 def _stream(stream) -> int:
     if stream is None:
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # the handle without a Stream object around it
+        return raw(torch.cuda.current_device()) if raw else torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -282,11 +283,11 @@ def commit_step(table: Sequence[TensorEntry] | PreparedTable, step: int, hparams
     hp = _hp(hparams)
     if zero_grad:
         _check(library().apc_commit_step_ex(ctypes.addressof(arr), n, ctypes.addressof(hp), int(step),
-                                            COMMIT_ZERO_GRAD, ctypes.c_void_p(_stream(stream)),
-                                            ctypes.c_void_p(_ptr(out, 8))))
+                                            COMMIT_ZERO_GRAD, _stream(stream),
+                                            _ptr(out, 8)))
     else:
         _check(library().apc_commit_step(ctypes.addressof(arr), n, ctypes.addressof(hp), int(step),
-                                         ctypes.c_void_p(_stream(stream)), ctypes.c_void_p(_ptr(out, 8))))
+                                         _stream(stream), _ptr(out, 8)))
     return out
 
 
@@ -298,8 +299,8 @@ def commit_step_bf16(table: Sequence[TensorEntryBF16] | PreparedTable, step: int
     out = _out(out, 3, first)
     hp = _hp(hparams)
     _check(library().apc_commit_step_bf16(ctypes.addressof(arr), n, ctypes.addressof(hp), int(step),
-                                          COMMIT_ZERO_GRAD if zero_grad else 0, ctypes.c_void_p(_stream(stream)),
-                                          ctypes.c_void_p(_ptr(out, 8))))
+                                          COMMIT_ZERO_GRAD if zero_grad else 0, _stream(stream),
+                                          _ptr(out, 8)))
     return out
 
 
@@ -339,8 +340,8 @@ def digest(buffers: Iterable[BufferEntry] | PreparedTable, num_slots: int = 4, s
     tensor."""
     arr, n, first = _buffers(buffers)
     out = _out(out, num_slots, first)
-    _check(library().apc_digest(ctypes.addressof(arr), n, int(num_slots), ctypes.c_void_p(_stream(stream)),
-                                ctypes.c_void_p(_ptr(out, 8))))
+    _check(library().apc_digest(ctypes.addressof(arr), n, int(num_slots), _stream(stream),
+                                _ptr(out, 8)))
     return out
 
 
@@ -349,8 +350,8 @@ def count_nonzero(buffers: Iterable[BufferEntry] | PreparedTable, num_slots: int
     of nonzero words.  Returns the device int64[num_slots] output tensor."""
     arr, n, first = _buffers(buffers)
     out = _out(out, num_slots, first)
-    _check(library().apc_count_nonzero(ctypes.addressof(arr), n, int(num_slots), ctypes.c_void_p(_stream(stream)),
-                                       ctypes.c_void_p(_ptr(out, 8))))
+    _check(library().apc_count_nonzero(ctypes.addressof(arr), n, int(num_slots), _stream(stream),
+                                       _ptr(out, 8)))
     return out
 
 
@@ -403,7 +404,7 @@ def upload(segments: Iterable[Segment] | PreparedTable, max_ctas: int = 0, strea
     """Enqueue the SM-driven host-to-device upload of ``segments`` on at
     most ``max_ctas`` CTAs (``apc_upload``; 0 = one per SM)."""
     arr, n = _segments(segments)
-    _check(library().apc_upload(ctypes.addressof(arr), n, int(max_ctas), ctypes.c_void_p(_stream(stream))))
+    _check(library().apc_upload(ctypes.addressof(arr), n, int(max_ctas), _stream(stream)))
 
 
 def set_reserved_sms(n: int) -> None:
@@ -434,7 +435,7 @@ def device_status() -> int:
 def selftest_wait_timeout(limit_ns: int, stream=None) -> None:
     """Launch the bounded-wait self-test: a wait that nothing completes gives
     up after ``limit_ns`` and records APC_ETIMEOUT for :func:`device_status`."""
-    _check(library().apc_selftest_wait_timeout(int(limit_ns), ctypes.c_void_p(_stream(stream))))
+    _check(library().apc_selftest_wait_timeout(int(limit_ns), _stream(stream)))
 
 
 def state_buffers(p, m, v, w, global_offset: int = 0) -> list[BufferEntry]:
