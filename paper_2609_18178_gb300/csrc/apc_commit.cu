@@ -179,16 +179,17 @@ struct F32State {
   template <bool ZERO>
   __device__ static void mis_pair(const StageDesc &sd, const Mis &x, uint32_t e, const Scalars &s, Acc &a) {
     const uint32_t f = e + kConsumers;
-    float p0 = x.p[e], p1 = x.p[f], m0 = x.m[e], m1 = x.m[f], v0 = x.v[e], v1 = x.v[f];
-    uint32_t w0, w1;
-    adamw_pair(p0, p1, m0, m1, v0, v1, x.g[e], x.g[f], s, w0, w1);
-    mis_store<ZERO>(sd, e, p0, m0, v0, w0);
-    mis_store<ZERO>(sd, f, p1, m1, v1, w1);
+    float p[2] = {x.p[e], x.p[f]}, m[2] = {x.m[e], x.m[f]}, v[2] = {x.v[e], x.v[f]};
+    const uint32_t gw[2] = {x.g[e], x.g[f]};
+    adamw_group<2>(p, m, v, gw, s);
+    const uint32_t w = pack_bf16x2(p[0], p[1]);
+    mis_store<ZERO>(sd, e, p[0], m[0], v[0], w & 0xFFFFu);
+    mis_store<ZERO>(sd, f, p[1], m[1], v[1], w >> 16);
     const uint32_t G = sd.G + e;
-    a.p += digest_term<0>(G, __float_as_uint(p0), s.one) + digest_term<kConsumers>(G, __float_as_uint(p1), s.one);
-    a.m += digest_term<0>(G, __float_as_uint(m0), s.one) + digest_term<kConsumers>(G, __float_as_uint(m1), s.one);
-    a.v += digest_term<0>(G, __float_as_uint(v0), s.one) + digest_term<kConsumers>(G, __float_as_uint(v1), s.one);
-    a.w += digest_term<0>(G, w0, s.one) + digest_term<kConsumers>(G, w1, s.one);
+    a.p += digest_term<0>(G, __float_as_uint(p[0]), s.one) + digest_term<kConsumers>(G, __float_as_uint(p[1]), s.one);
+    a.m += digest_term<0>(G, __float_as_uint(m[0]), s.one) + digest_term<kConsumers>(G, __float_as_uint(m[1]), s.one);
+    a.v += digest_term<0>(G, __float_as_uint(v[0]), s.one) + digest_term<kConsumers>(G, __float_as_uint(v[1]), s.one);
+    a.w += digest_term<0>(G, w & 0xFFFFu, s.one) + digest_term<kConsumers>(G, w >> 16, s.one);
   }
 
   // Element e of a misaligned tile.
@@ -214,20 +215,21 @@ struct F32State {
 
   // Four consecutive elements at the compile-time element offset OFF from
   // the thread's output addresses, whose first element has digest index G.
-  template <uint32_t OFF, bool PAIRED>
+  template <uint32_t OFF, bool ZERO>
   __device__ static void compute_store(const Dst &d, uint32_t G, const Regs &r, const Scalars &s, Acc &a) {
     constexpr uint32_t off = OFF;
     float p[4] = {r.p.x, r.p.y, r.p.z, r.p.w};
     float m[4] = {r.m.x, r.m.y, r.m.z, r.m.w};
     float v[4] = {r.v.x, r.v.y, r.v.z, r.v.w};
     const uint32_t gw[4] = {r.g.x & 0xFFFFu, r.g.x >> 16, r.g.y & 0xFFFFu, r.g.y >> 16};
-    if constexpr (PAIRED) {
-      uint32_t unused[4];
-      adamw_pair(p[0], p[1], m[0], m[1], v[0], v[1], gw[0], gw[1], s, unused[0], unused[1]);
-      adamw_pair(p[2], p[3], m[2], m[3], v[2], v[3], gw[2], gw[3], s, unused[2], unused[3]);
-    } else {
+    if constexpr (ZERO) {
+      // bound by its 30 bytes per element: the grouped form, with fewer
+      // instructions, measured slower here (453 M elements in 2,150 us
+      // against 2,043)
 #pragma unroll
       for (int j = 0; j < 4; ++j) (void)adamw_element(p[j], m[j], v[j], gw[j], s);
+    } else {
+      adamw_group<4>(p, m, v, gw, s);
     }
     __stcs(reinterpret_cast<float4 *>(static_cast<float *>(d.p) + off), make_float4(p[0], p[1], p[2], p[3]));
     __stcs(reinterpret_cast<float4 *>(static_cast<float *>(d.m) + off), make_float4(m[0], m[1], m[2], m[3]));
@@ -313,11 +315,11 @@ struct BF16State {
   template <bool ZERO>
   __device__ static void mis_pair(const StageDesc &sd, const Mis &x, uint32_t e, const Scalars &s, Acc &a) {
     const uint32_t f = e + kConsumers;
-    float p0 = bf16_value(x.p[e]), p1 = bf16_value(x.p[f]), m0 = bf16_value(x.m[e]), m1 = bf16_value(x.m[f]);
-    float v0 = bf16_value(x.v[e]), v1 = bf16_value(x.v[f]);
-    uint32_t unused0, unused1;
-    adamw_pair(p0, p1, m0, m1, v0, v1, x.g[e], x.g[f], s, unused0, unused1);
-    const uint32_t p = pack_bf16x2(p0, p1), m = pack_bf16x2(m0, m1), v = pack_bf16x2(v0, v1);
+    float pf[2] = {bf16_value(x.p[e]), bf16_value(x.p[f])}, mf[2] = {bf16_value(x.m[e]), bf16_value(x.m[f])};
+    float vf[2] = {bf16_value(x.v[e]), bf16_value(x.v[f])};
+    const uint32_t gw[2] = {x.g[e], x.g[f]};
+    adamw_group<2>(pf, mf, vf, gw, s);
+    const uint32_t p = pack_bf16x2(pf[0], pf[1]), m = pack_bf16x2(mf[0], mf[1]), v = pack_bf16x2(vf[0], vf[1]);
     mis_store<ZERO>(sd, e, p & 0xFFFFu, m & 0xFFFFu, v & 0xFFFFu);
     mis_store<ZERO>(sd, f, p >> 16, m >> 16, v >> 16);
     const uint32_t G = sd.G + e;
@@ -345,7 +347,7 @@ struct BF16State {
     if (ZERO) __stcs(sd.g + e, (uint16_t)0);
   }
 
-  template <uint32_t OFF, bool PAIRED>
+  template <uint32_t OFF, bool ZERO>
   __device__ static void compute_store(const Dst &d, uint32_t G, const Regs &r, const Scalars &s, Acc &a) {
     constexpr uint32_t off = OFF;
     const uint32_t pw[4] = {r.p.x & 0xFFFFu, r.p.x >> 16, r.p.y & 0xFFFFu, r.p.y >> 16};
@@ -353,25 +355,13 @@ struct BF16State {
     const uint32_t vw[4] = {r.v.x & 0xFFFFu, r.v.x >> 16, r.v.y & 0xFFFFu, r.v.y >> 16};
     const uint32_t gw[4] = {r.g.x & 0xFFFFu, r.g.x >> 16, r.g.y & 0xFFFFu, r.g.y >> 16};
     float pf[4], mf[4], vf[4];
-    if constexpr (PAIRED) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        pf[j] = bf16_value(pw[j]);
-        mf[j] = bf16_value(mw[j]);
-        vf[j] = bf16_value(vw[j]);
-      }
-      uint32_t unused[4];
-      adamw_pair(pf[0], pf[1], mf[0], mf[1], vf[0], vf[1], gw[0], gw[1], s, unused[0], unused[1]);
-      adamw_pair(pf[2], pf[3], mf[2], mf[3], vf[2], vf[3], gw[2], gw[3], s, unused[2], unused[3]);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        pf[j] = bf16_value(pw[j]);
-        mf[j] = bf16_value(mw[j]);
-        vf[j] = bf16_value(vw[j]);
-        (void)adamw_element(pf[j], mf[j], vf[j], gw[j], s);
-      }
+    for (int j = 0; j < 4; ++j) {
+      pf[j] = bf16_value(pw[j]);
+      mf[j] = bf16_value(mw[j]);
+      vf[j] = bf16_value(vw[j]);
     }
+    adamw_group<4>(pf, mf, vf, gw, s);
     const uint32_t p01 = pack_bf16x2(pf[0], pf[1]), p23 = pack_bf16x2(pf[2], pf[3]);
     const uint32_t m01 = pack_bf16x2(mf[0], mf[1]), m23 = pack_bf16x2(mf[2], mf[3]);
     const uint32_t v01 = pack_bf16x2(vf[0], vf[1]), v23 = pack_bf16x2(vf[2], vf[3]);
@@ -420,10 +410,7 @@ __device__ __forceinline__ void store_groups(const Dst &d, uint32_t G1, const ty
   constexpr uint32_t off = (uint32_t)(K * L::kConsumers) * 4;
   if (ok[K]) {
     if (ZERO) __stcs(reinterpret_cast<uint2 *>(d.g + off), make_uint2(0u, 0u));
-    // the gradient-zeroing pass is bound by its 30 bytes per element, and the
-    // packed multiplies measured slower there (33.9 against 33.5 ms on the
-    // full model): it keeps one element at a time
-    L::template compute_store<off, APC_PAIRED_ADAMW != 0 && !ZERO>(d, G1, r[K], s, a);
+    L::template compute_store<off, ZERO>(d, G1, r[K], s, a);
   }
   if constexpr (K + 1 < L::kGroups) store_groups<L, ZERO, K + 1>(d, G1, r, ok, s, a);
 }
@@ -511,7 +498,7 @@ __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
   Acc a{0, 0, 0, 0};
   if (warp == L::kConsumerWarps) {
     // ------------------------------------------------------------ producer
-    const Scalars s{plan.h, plan.one};
+    const Scalars s{plan.h, plan.pair, plan.limit, plan.one};
     uint32_t phase = 0;
     int stage = 0;
     uint64_t issued = 0;
@@ -588,7 +575,7 @@ __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
     __syncwarp();
   } else {
     // ----------------------------------------------------------- consumers
-    const Scalars s{plan.h, plan.one};
+    const Scalars s{plan.h, plan.pair, plan.limit, plan.one};
     const int ct = threadIdx.x;  // 0 .. L::kConsumers-1
     uint32_t phase = 0;
     int stage = 0;

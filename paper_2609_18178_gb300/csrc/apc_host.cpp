@@ -298,13 +298,33 @@ uint32_t commit_launch_tile(const apc::CommitEntry *e, size_t count, uint64_t fu
   return (uint32_t)best;
 }
 
+// The scalars of a launch, and the constants of adamw_group with the bounds
+// that its form needs of them: den >= eps >= 2^-50 keeps a / den below 2^121;
+// 1/sqrt(bc2) <= 2^16 keeps the root of its 2^-126 addend out of den; a
+// nonzero step in [2^-60, 2^20] keeps step * 2^-64 normal and a subnormal
+// quotient's term below 2^-106.
+template <int MAXE>
+void commit_scalars(const float h[8], apc::CommitPlan<MAXE> *plan) {
+  std::memcpy(plan->h, h, sizeof plan->h);
+  const float pairs[apc::kPairs] = {h[0],     h[1],       h[2],       h[3], h[5], -h[7] * 0x1p-32f, h[6] * 0x1p-64f,
+                                    -0x1p64f, -0x1p-126f, 0.5f, 1.0f};
+  for (int k = 0; k < apc::kPairs; ++k) {
+    uint32_t bits;
+    std::memcpy(&bits, &pairs[k], sizeof bits);
+    plan->pair[k] = (uint64_t)bits << 32 | bits;
+  }
+  const bool fits = h[4] >= 0x1p-50f && h[7] >= 1.0f && h[7] <= 0x1p16f &&
+                    (h[6] == 0.0f || (h[6] >= 0x1p-60f && h[6] <= 0x1p20f));
+  plan->limit = fits ? 128.0f : -1.0f;
+}
+
 // Entries arrive without tile_begin; each batch places their tiles.
 template <int MAXE, typename Launch>
 apc_status run_commit_batches(const std::vector<apc::CommitEntry> &entries, const float h[8], int layout,
                               bool zero_grad, unsigned grid_cap, void *stream, unsigned long long *out,
                               Launch launch) {
   std::unique_ptr<apc::CommitPlan<MAXE>> plan(new apc::CommitPlan<MAXE>);  // not cleared: the kernel reads what is filled
-  std::memcpy(plan->h, h, sizeof plan->h);
+  commit_scalars(h, plan.get());
   plan->one = 1;
   size_t i = 0;
   while (i < entries.size()) {

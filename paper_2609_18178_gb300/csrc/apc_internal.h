@@ -81,11 +81,6 @@ constexpr int kCommitBlocksPerSm = APC_COMMIT_BLOCKS_PER_SM;
 #ifndef APC_COMMIT_CONTIGUOUS
 #define APC_COMMIT_CONTIGUOUS 1
 #endif
-// AdamW's multiplies as packed two-lane binary32 instructions over pairs of
-// elements (1), or one element at a time (0); the bits are the same.
-#ifndef APC_PAIRED_ADAMW
-#define APC_PAIRED_ADAMW 1
-#endif
 // A stage holds one tile of p, m, v and g: 14 bytes per element for fp32
 // state (66.5 KB, 200 KB per CTA at the defaults), 8 for bf16 state (81 KB,
 // 162 KB per CTA).
@@ -118,14 +113,28 @@ struct CommitEntry {
   uint16_t mis;
 };
 
+// Constants of the commit kernel's packed operations, each in both lanes.
+enum CommitPair {
+  kPairB1, kPair1B1, kPairB2, kPair1B2,  // b1, 1-b1, b2, 1-b2
+  kPairDecay,                            // 1-lr*wd
+  kPairRsb2,                             // -1/sqrt(bc2) * 2^-32
+  kPairStep,                             // lr/bc1 * 2^-64
+  kPairNeg64, kPairNegTiny,              // -2^64, -2^-126
+  kPairHalf, kPairOne,                   // 1/2, 1
+  kPairs
+};
+
 template <int MAXE>
 struct CommitPlan {
   float h[8];            // b1, 1-b1, b2, 1-b2, eps, 1-lr*wd, lr/bc1, 1/sqrt(bc2)
+  uint64_t pair[kPairs];
+  float limit;           // adamw_group's bound, -1 where its form does not apply
+  uint32_t pad_;
   uint64_t total_tiles;
   uint32_t count;
   uint32_t one;          // 1: the FMA-pipe carry-add multiplier of the digest
   uint32_t tile;         // elements per tile of this launch (a multiple of 64, at most commit_tile)
-  uint32_t pad_;
+  uint32_t pad2_;
   CommitEntry e[MAXE];
 };
 

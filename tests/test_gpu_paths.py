@@ -201,3 +201,66 @@ def test_commit_launch_tiles(monkeypatch, layout, limit):
         shifts[(1, "g")] = 1
         committed(tensors[:1], [77], 2, layout, False, shifts)
         committed(tensors, [77] * 4, 2, layout, True, shifts)
+
+
+def any_floats(rng, n, f32):
+    """Finite words of every exponent, signs and zeros among them, runs of one
+    magnitude beside runs of mixed ones."""
+    if f32:
+        a = rng.integers(0, 2**32, size=n, dtype=np.uint64).astype(np.uint32)
+        e = np.where(np.arange(n) // 64 % 3 == 0, rng.integers(0, 255, size=n),
+                     np.repeat(rng.integers(0, 255, size=n // 16 + 1), 16)[:n]).astype(np.uint32)
+        a = (a & np.uint32(0x807FFFFF)) | (e << np.uint32(23))
+    else:
+        a = rng.integers(0, 2**16, size=n, dtype=np.uint64).astype(np.uint16)
+        e = np.where(np.arange(n) // 64 % 3 == 0, rng.integers(0, 255, size=n),
+                     np.repeat(rng.integers(0, 255, size=n // 16 + 1), 16)[:n]).astype(np.uint16)
+        a = (a & np.uint16(0x807F)) | (e << np.uint16(7))
+    a[rng.random(n) < 0.05] = 0
+    a[rng.random(n) < 0.02] = 0x80000000 if f32 else 0x8000
+    return a
+
+
+@pytest.mark.parametrize("layout", ["f32", "bf16"])
+@pytest.mark.parametrize("hp,step", [
+    (dict(), 1), (dict(), 1000), (dict(eps=1e-15), 2), (dict(eps=2.0**-50), 3), (dict(eps=1e-30), 3), (dict(eps=300.0), 1),
+    (dict(lr=0.0), 5), (dict(lr=1e-25), 5), (dict(lr=1e-18), 5), (dict(lr=1e7), 5), (dict(beta2=0.9999999999), 1),
+    (dict(beta1=0.0, beta2=0.0), 1), (dict(weight_decay=0.0), 18)])
+def test_update_over_all_magnitudes(layout, hp, step):
+    """The grouped square root and quotient, and their fallback, on states of
+    every magnitude: subnormal, zero of either sign, tiny beside ordinary, and
+    so large that squares overflow.  Results that overflow or are not numbers
+    are compared as such; everything else bit by bit."""
+    rng = np.random.default_rng(step)
+    f32, n = layout == "f32", 120_011
+    hp = dict(oracle.DEFAULT_HP, **hp)
+    w = {k: any_floats(rng, n, f32) for k in "pmv"}
+    w["v"] &= w["v"].dtype.type(0x7FFFFFFF if f32 else 0x7FFF)
+    w["g"] = any_floats(rng, n, False)
+    ordinary = np.arange(n) // 5000 % 2 == 0      # half of it in a job's own range
+    p, m, v = (synth.state if f32 else synth.state_bf16)(n, 0)
+    for k, a in (("p", p), ("m", m), ("v", v), ("g", synth.grad(n, 0, 1))):
+        a = a.view(w[k].dtype)
+        w[k] = np.where(ordinary & (rng.random(n) < 0.9), a, w[k])
+    ref = {k: w[k].copy() for k in "pmv"}
+    d = {k: dev_words(w[k]) for k in w}
+    h8 = oracle.resolve_hparams(hp, step)
+    if f32:
+        d["w"] = torch.zeros(n, dtype=torch.int16, device="cuda")
+        out = apc.commit_step([apc.TensorEntry(d["p"], d["m"], d["v"], d["g"], d["w"], 9)], step, hp)
+        f = {k: ref[k].view(np.float32) for k in "pmv"}
+        ref["w"], _ = oracle.commit(f["p"], f["m"], f["v"], w["g"], 9, h8)
+        ver = apc.digest(apc.state_buffers(d["p"], d["m"], d["v"], d["w"], 9), 4)
+    else:
+        out = apc.commit_step_bf16([apc.TensorEntryBF16(d["p"], d["m"], d["v"], d["g"], 9)], step, hp)
+        oracle.commit_bf16(ref["p"], ref["m"], ref["v"], w["g"], 9, h8)
+        ver = apc.digest(apc.state_buffers_bf16(d["p"], d["m"], d["v"], 9), 3)
+    for k in ref:
+        got = d[k].cpu().numpy().view(ref[k].dtype)
+        top = 0x7F800000 if got.itemsize == 4 else 0x7F80
+        mask = 0x7FFFFFFF if got.itemsize == 4 else 0x7FFF
+        nan_g, nan_r = (got & mask) > top, (ref[k] & mask) > top
+        assert np.array_equal(nan_g, nan_r), k
+        bad = np.nonzero((got != ref[k]) & ~nan_r)[0]
+        assert bad.size == 0, (k, bad[:5], got[bad[:5]], ref[k][bad[:5]])
+    assert apc.digests_to_host(out) == apc.digests_to_host(ver)
