@@ -339,4 +339,25 @@ __device__ __forceinline__ uint64_t warp_sum(uint64_t x) {
   return x;
 }
 
+// Add a warp's running sums to its slot of the CTA's and clear them (slot -1: none yet).
+__device__ __forceinline__ void flush(uint64_t &acc, int slot, unsigned long long *s_acc) {
+  const uint64_t x = warp_sum(acc);
+  if ((threadIdx.x & 31) == 0 && slot >= 0 && x) atomicAdd(&s_acc[slot], (unsigned long long)x);
+  acc = 0;
+}
+
+// The entry whose tiles hold `tile`, at or after entry `lo` (the last one that
+// begins at or before it: an entry without full tiles begins where the next
+// one does).
+template <int MAXE>
+__device__ __forceinline__ uint32_t entry_of(const DigestPlan<MAXE> &plan, uint32_t lo, uint64_t tile) {
+  uint32_t hi = plan.count;  // e[lo].tile_begin <= tile, e[hi] beyond
+  while (hi - lo > 1) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (plan.e[mid].tile_begin <= tile) lo = mid;
+    else hi = mid;
+  }
+  return lo;
+}
+
 }  // namespace apc

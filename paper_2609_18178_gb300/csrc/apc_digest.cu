@@ -210,26 +210,6 @@ __device__ __forceinline__ void cp16(uint32_t dst, const void *src) {
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_wait_all_but_newest() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 
-__device__ __forceinline__ void flush(uint64_t &acc, int slot, unsigned long long *s_acc) {
-  const uint64_t x = warp_sum(acc);
-  if ((threadIdx.x & 31) == 0 && slot >= 0 && x) atomicAdd(&s_acc[slot], (unsigned long long)x);
-  acc = 0;
-}
-
-// The entry whose tiles hold `tile`, at or after entry `lo` (the last one that
-// begins at or before it: an entry without full tiles begins where the next
-// one does).
-template <int MAXE>
-__device__ __forceinline__ uint32_t entry_of(const DigestPlan<MAXE> &plan, uint32_t lo, uint64_t tile) {
-  uint32_t hi = plan.count;  // e[lo].tile_begin <= tile, e[hi] beyond
-  while (hi - lo > 1) {
-    const uint32_t mid = (lo + hi) >> 1;
-    if (plan.e[mid].tile_begin <= tile) lo = mid;
-    else hi = mid;
-  }
-  return lo;
-}
-
 // One walk: the warps' tiles of the fp32 entries (T32) or of the bf16 entries.
 // Each kind's tiles are shared out over all CTAs on their own: a bf16 tile
 // costs less than an fp32 one, and a CTA with tiles of one kind only would

@@ -350,7 +350,7 @@ apc_status run_commit_batches(const std::vector<apc::CommitEntry> &entries, cons
 }
 
 // Entries arrive with the element count of their vector body in tile_begin;
-// tiles_of(body) is the kernel's tile count of an entry.
+// tiles_of(body, element size) is the kernel's count of whole tiles in it.
 template <int MAXE, typename Tiles, typename Launch>
 apc_status run_digest_batches(const std::vector<apc::DigestEntry> &entries, unsigned grid_cap, Tiles tiles_of,
                               Launch launch, const char *what) {
@@ -362,7 +362,7 @@ apc_status run_digest_batches(const std::vector<apc::DigestEntry> &entries, unsi
     uint64_t tiles = 0, tiles32 = 0;
     for (size_t j = 0; j < k; ++j) {
       apc::DigestEntry e = entries[i + j];
-      const uint64_t t = tiles_of(e.tile_begin);
+      const uint64_t t = tiles_of(e.tile_begin, e.dtype == APC_F32 ? 4 : 2);
       e.tile_begin = tiles;
       tiles += t;
       if (e.dtype == APC_F32) tiles32 = tiles;
@@ -591,7 +591,7 @@ APC_EXPORT apc_status apc_digest(const apc_buffer *bufs, int32_t num_bufs, int32
   const uint64_t launches = ceil_div(entries.size(), small ? apc::kDigestSmall : apc::kDigestLarge);
   const int u = body / apc::digest_tile(apc::kDigestLong) >= apc::kDigestLongTiles * warps * launches ? apc::kDigestLong
                                                                                                        : apc::kDigestShort;
-  const auto tiles_of = [u](uint64_t n) { return n / apc::digest_tile(u); };
+  const auto tiles_of = [u](uint64_t n, uint64_t) { return n / apc::digest_tile(u); };
   if (small)
     return run_digest_batches<apc::kDigestSmall>(
         entries, cap, tiles_of, [&](const auto &plan, unsigned grid) { return apc::launch_digest_small(plan, u, grid, stream, out); },
@@ -613,7 +613,7 @@ APC_EXPORT apc_status apc_count_nonzero(const apc_buffer *bufs, int32_t num_bufs
   Device d;
   if ((st = device_info(&d)) != APC_OK) return st;
   unsigned long long *out = reinterpret_cast<unsigned long long *>(out_counts);
-  const auto tiles_of = [](uint64_t n) { return std::max<uint64_t>(1, ceil_div(n, apc::kCountTile)); };
+  const auto tiles_of = [](uint64_t n, uint64_t es) { return n * es / apc::kCountTileBytes; };
   if (entries.size() <= (size_t)apc::kDigestSmall)
     return run_digest_batches<apc::kDigestSmall>(
         entries, grid_for(UINT64_MAX, d.sms, d.count_small), tiles_of,

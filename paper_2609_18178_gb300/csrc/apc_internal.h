@@ -165,20 +165,19 @@ constexpr int kDigestShort = 2, kDigestLong = 4;  // U: vectors per lane per til
 constexpr uint64_t kDigestLongTiles = 8;
 constexpr uint64_t digest_tile(int u) { return (uint64_t)32 * kVec * u; }  // elements: 512 and 1,024
 
-// Guard (count) kernel: the same plans and tiling scheme with its own shape;
-// one compare per word leaves it bound by HBM, so its shape is set by the
-// bytes each SM keeps in flight: one CTA of 1024 threads per SM with 4
-// vectors each (64 KB of bf16 words) reaches 99% of the copy rate, where
-// three CTAs of 384 x 3 reached 96%.
+// Guard (count) kernel: the same plans and walk with tiles of its own; one
+// compare per word leaves it bound by HBM, so its shape is set by the bytes
+// each SM keeps in flight: 6 loads a lane (96 KB per SM) read 14.5 GB in
+// 1,972 us, 4 in 2,024, 8 in 1,987 (2,001 with 512 threads), 2 in 2,037.
 #ifndef APC_COUNT_THREADS
 #define APC_COUNT_THREADS 1024
 #endif
-#ifndef APC_COUNT_UNROLL
-#define APC_COUNT_UNROLL 4
+#ifndef APC_COUNT_GROUPS
+#define APC_COUNT_GROUPS 6
 #endif
 constexpr int kCountThreads = APC_COUNT_THREADS;
-constexpr int kCountUnroll = APC_COUNT_UNROLL;
-constexpr uint64_t kCountTile = (uint64_t)kCountThreads * kVec * kCountUnroll;  // 32,768 elements
+constexpr int kCountGroups = APC_COUNT_GROUPS;                   // 16-byte loads per lane per tile
+constexpr uint32_t kCountTileBytes = 32 * 16 * kCountGroups;     // one warp's tile
 // Minimum resident CTAs per SM the digest kernel is compiled for (its
 // register cap: 65,536 / (threads x this)), and extra dynamic shared memory
 // per CTA beyond its stages (0 by default; a larger CTA footprint keeps two
@@ -192,9 +191,9 @@ constexpr uint64_t kCountTile = (uint64_t)kCountThreads * kVec * kCountUnroll;  
 
 // One buffer of the digest kernel (32 bytes).
 //   head: scalar elements before the first 16-byte boundary (<= 7); then
-//         8-element vectors in tiles (digest_tile(U) elements, full ones
-//         only, for the digest kernel; kCountTile for the count kernel); then a
-//         scalar tail.
+//         8-element vectors, the whole tiles of which (digest_tile(U) elements
+//         for the digest kernel, kCountTileBytes for the count kernel) are
+//         counted in tile_begin; then a scalar tail.
 struct DigestEntry {
   const void *data;
   uint64_t n;

@@ -264,3 +264,28 @@ def test_update_over_all_magnitudes(layout, hp, step):
         bad = np.nonzero((got != ref[k]) & ~nan_r)[0]
         assert bad.size == 0, (k, bad[:5], got[bad[:5]], ref[k][bad[:5]])
     assert apc.digests_to_host(out) == apc.digests_to_host(ver)
+
+
+@pytest.mark.parametrize("limit", [None, 1])
+def test_guard_warp_tiles(monkeypatch, limit):
+    """Counts over buffers of no, one and several of the guard's 3,072-byte
+    warp tiles with every remainder, types and slots mixed: single nonzero
+    words at the edges, and dense ones."""
+    grid_limit(monkeypatch, limit)
+    rng = np.random.default_rng(17)
+    bufs, want, keep = [], [0] * 8, []
+    for i, nbytes in enumerate([4, 12, 16, 60, 512, 3056] + [k * 3072 + d for k in (1, 2, 33) for d in (-16, -4, 0, 4, 16, 500)]):
+        for f32 in (True, False):
+            n, shift = nbytes // (4 if f32 else 2), int(rng.integers(0, 8))
+            a = words(rng, n + shift, f32)
+            if i % 2:
+                a[:] = 0
+                a[shift + rng.integers(0, n, size=3)] = 1
+                a[shift] = a[-1] = 1
+            a[:shift] = 7                      # before the buffer: not counted
+            slot = (3 * i + f32) % 8
+            want[slot] += int(np.count_nonzero(a[shift:]))
+            keep.append(dev_words(a))
+            bufs.append(apc.BufferEntry(keep[-1][shift:], slot, 0, apc.F32 if f32 else apc.BF16))
+            assert apc.digests_to_host(apc.count_nonzero([bufs[-1]], 8))[slot] == np.count_nonzero(a[shift:])
+    assert apc.digests_to_host(apc.count_nonzero(bufs, 8)) == want
