@@ -346,11 +346,11 @@ __device__ __forceinline__ void flush(uint64_t &acc, int slot, unsigned long lon
   acc = 0;
 }
 
-// The entry whose tiles hold `tile`, at or after entry `lo` (the last one that
-// begins at or before it: an entry without full tiles begins where the next
-// one does).
-template <int MAXE>
-__device__ __forceinline__ uint32_t entry_of(const DigestPlan<MAXE> &plan, uint32_t lo, uint64_t tile) {
+// The entry of a launch plan whose tiles hold `tile`, at or after entry `lo`
+// (the last one that begins at or before it: an entry without tiles begins
+// where the next one does).
+template <class Plan>
+__device__ __forceinline__ uint32_t entry_of(const Plan &plan, uint32_t lo, uint64_t tile) {
   uint32_t hi = plan.count;  // e[lo].tile_begin <= tile, e[hi] beyond
   while (hi - lo > 1) {
     const uint32_t mid = (lo + hi) >> 1;

@@ -693,10 +693,12 @@ APC_EXPORT apc_status apc_upload(const apc_segment *segs, int32_t num_segments, 
     e.src = static_cast<const uint8_t *>(src);
     e.bytes = g.bytes;
     const uintptr_t d = (uintptr_t)e.dst, s = (uintptr_t)e.src;
-    const uint64_t head = (16 - (d & 15)) & 15;
-    e.body = ((d ^ s) & 15) == 0 && g.bytes > head ? (g.bytes - head) & ~(uint64_t)15 : 0;
-    e.tile_begin = (e.body + apc::kUploadTile - 1) / apc::kUploadTile;  // tile count until placed
-    e.scalar_begin = g.bytes - e.body;                                  // scalar count until placed
+    const bool aligned = ((d ^ s) & 15) == 0;
+    const uint64_t h0 = (16 - (d & 15)) & 15;  // bytes before the destination's first 16-byte boundary
+    const uint64_t head = aligned || h0 == 15 ? h0 : h0 + 16, tail = aligned ? 0 : 16;
+    e.body = g.bytes > head + tail ? (g.bytes - head - tail) & ~(uint64_t)15 : 0;
+    e.head = (uint32_t)(e.body ? head : std::min<uint64_t>(g.bytes, 64));
+    e.shift = e.body ? (uint32_t)((s + head) & 15) : 0;
     entries.push_back(e);
   }
   // destinations must not overlap each other or any source (sorted sweep)
@@ -712,24 +714,20 @@ APC_EXPORT apc_status apc_upload(const apc_segment *segs, int32_t num_segments, 
   apc_status st = device_info(&d);
   if (st != APC_OK) return st;
   const unsigned cap = max_ctas > 0 ? (unsigned)max_ctas : (unsigned)d.sms;
-  auto plan = std::make_unique<apc::UploadPlan<apc::kUploadMax>>();
+  std::unique_ptr<apc::UploadPlan<apc::kUploadMax>> plan(new apc::UploadPlan<apc::kUploadMax>);
   size_t i = 0;
   while (i < entries.size()) {
     const size_t k = std::min(entries.size() - i, (size_t)apc::kUploadMax);
-    uint64_t tiles = 0, scalars = 0;
+    uint64_t tiles = 0;
     for (size_t j = 0; j < k; ++j) {
       apc::UploadEntry e = entries[i + j];
-      const uint64_t t = e.tile_begin, c = e.scalar_begin;
       e.tile_begin = tiles;
-      e.scalar_begin = scalars;
-      tiles += t;
-      scalars += c;
+      tiles += e.body / apc::kUploadTile;
       plan->e[j] = e;
     }
     plan->count = (uint32_t)k;
     plan->total_tiles = tiles;
-    plan->total_scalar = scalars;
-    const uint64_t want = std::max<uint64_t>(tiles, (scalars + apc::kUploadThreads - 1) / apc::kUploadThreads);
+    const uint64_t want = std::max<uint64_t>(tiles, k);
     const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(want, cap));
     int e = apc::launch_upload(*plan, grid, stream);
     if (e) return cuda_fail(e, "upload kernel launch");

@@ -289,3 +289,29 @@ def test_guard_warp_tiles(monkeypatch, limit):
             bufs.append(apc.BufferEntry(keep[-1][shift:], slot, 0, apc.F32 if f32 else apc.BF16))
             assert apc.digests_to_host(apc.count_nonzero([bufs[-1]], 8))[slot] == np.count_nonzero(a[shift:])
     assert apc.digests_to_host(apc.count_nonzero(bufs, 8)) == want
+
+
+@pytest.mark.parametrize("ctas", [0, 1])
+def test_upload_every_relative_offset(ctas):
+    """Segments at every offset of source against destination from a 16-byte
+    boundary, of sizes around the upload's words, remainders and 4 KB warp
+    tiles; every byte arrives and none outside the destinations changes."""
+    rng = np.random.default_rng(31)
+    sizes = list(range(1, 100)) + [k * 4096 + d for k in (1, 2, 17) for d in (-40, -16, 0, 1, 31, 47, 300)]
+    segs, want, total = [], [], 0
+    for i in range(256 * 3):
+        s, d = i % 16, i // 16 % 16
+        n = sizes[int(rng.integers(0, len(sizes)))]
+        segs.append((total + s, total + d, n))
+        total += (n + 16 + 63) // 64 * 64
+    host = torch.from_numpy(rng.integers(0, 256, size=total, dtype=np.uint8)).pin_memory()
+    dst = torch.full((total,), 0xEE, dtype=torch.uint8, device="cuda")
+    ref = np.full(total, 0xEE, np.uint8)
+    h = host.numpy()
+    for s, d, n in segs:
+        ref[d:d + n] = h[s:s + n]
+    apc.upload([apc.Segment(dst[d:d + n], host[s:s + n]) for s, d, n in segs], ctas)
+    assert np.array_equal(dst.cpu().numpy(), ref)
+    flat = torch.full_like(dst, 0xEE)            # and from device memory
+    apc.upload([apc.Segment(flat[d:d + n], dst[d:d + n]) for _, d, n in segs], ctas)
+    assert np.array_equal(flat.cpu().numpy(), ref)
