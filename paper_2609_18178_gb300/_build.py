@@ -41,7 +41,7 @@ PROBE_SRC = os.path.join(CSRC, "apc_probe.cu")
 
 def sources() -> list[str]:
     out = [os.path.join(CSRC, u) for u in UNITS]
-    out += [os.path.join(CSRC, h) for h in ("apc_internal.h", "apc_device.cuh", "apc_tma.cuh")]
+    out += [os.path.join(CSRC, h) for h in ("apc_internal.h", "apc_device.cuh", "apc_tma.cuh", "apc_launch.cuh")]
     out.append(os.path.join(INCLUDE, "apc.h"))
     return out
 

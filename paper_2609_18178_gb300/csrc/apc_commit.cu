@@ -59,6 +59,7 @@
 #include "../../include/apc.h"
 #include "apc_device.cuh"
 #include "apc_internal.h"
+#include "apc_launch.cuh"
 #include "apc_tma.cuh"
 
 namespace apc {
@@ -484,6 +485,7 @@ __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
   __shared__ uint64_t red[L::kDigests][L::kThreads / 32];
   __shared__ int abort_flag;
 
+  if (plan.more) chain_start_next();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < L::kStages; ++s) {
@@ -628,9 +630,11 @@ __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
 #pragma unroll
     for (int d = 0; d < L::kDigests; ++d) red[d][warp] = sums[d];
   __syncthreads();
-  if (warp < L::kDigests && !*(volatile int *)&abort_flag) {
+  if (warp < L::kDigests) {
+    const bool ok = !*(volatile int *)&abort_flag;
     const uint64_t r = warp_sum(lane < L::kThreads / 32 ? red[warp][lane] : 0);
-    if (lane == 0 && r) atomicAdd(&out[warp], (unsigned long long)r);
+    chain_wait();
+    if (ok && lane == 0 && r) atomicAdd(&out[warp], (unsigned long long)r);
   }
 }
 
@@ -670,9 +674,8 @@ template <class L, int MAXE, bool ZERO, bool MIS>
 int launch_t(const CommitPlan<MAXE> &plan, unsigned grid, void *stream, unsigned long long *out) {
   int e = ensure_smem_attribute<L, MAXE, ZERO, MIS>();
   if (e) return e;
-  commit_kernel<L, MAXE, ZERO, MIS>
-      <<<grid, L::kThreads, smem_bytes<L, MIS>(), (cudaStream_t)stream>>>(plan, out);
-  return (int)cudaGetLastError();
+  return launch_plan(commit_kernel<L, MAXE, ZERO, MIS>, plan, plan.chained, grid, L::kThreads, smem_bytes<L, MIS>(),
+                     stream, out);
 }
 
 template <class L, int MAXE>

@@ -332,6 +332,11 @@ __device__ __forceinline__ void acc_add(uint64_t &acc, uint64_t z, uint32_t one)
   acc = ((uint64_t)ahi << 32) | alo;
 }
 
+// The launches of one call form a chain (launch_plan): let the next one start,
+// and wait until the ones before have completed and their writes are visible.
+__device__ __forceinline__ void chain_start_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Sum of a warp's values, in every lane.
 __device__ __forceinline__ uint64_t warp_sum(uint64_t x) {
 #pragma unroll

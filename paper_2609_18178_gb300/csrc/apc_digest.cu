@@ -41,6 +41,7 @@
 #include "../../include/apc.h"
 #include "apc_device.cuh"
 #include "apc_internal.h"
+#include "apc_launch.cuh"
 
 namespace apc {
 namespace {
@@ -292,6 +293,7 @@ __global__ void __launch_bounds__(kThreads, APC_DIGEST_MIN_BLOCKS) digest_kernel
   __shared__ unsigned long long s_acc[APC_MAX_SLOTS];
   extern __shared__ __align__(16) uint4 stg[];
   const uint32_t stg_t = (uint32_t)__cvta_generic_to_shared(stg + threadIdx.x);  // this thread's slot 0, stage 0
+  if (plan.more) chain_start_next();
   if (threadIdx.x < APC_MAX_SLOTS) s_acc[threadIdx.x] = 0;
   __syncthreads();
   // what the entries hold beyond their full tiles, one entry per warp
@@ -302,7 +304,10 @@ __global__ void __launch_bounds__(kThreads, APC_DIGEST_MIN_BLOCKS) digest_kernel
   walk<true, U>(plan, stg, stg_t, s_acc);
   walk<false, U>(plan, stg, stg_t, s_acc);
   __syncthreads();
-  if (threadIdx.x < APC_MAX_SLOTS && s_acc[threadIdx.x]) atomicAdd(&out[threadIdx.x], s_acc[threadIdx.x]);
+  if (threadIdx.x < APC_MAX_SLOTS) {
+    chain_wait();
+    if (s_acc[threadIdx.x]) atomicAdd(&out[threadIdx.x], s_acc[threadIdx.x]);
+  }
 }
 
 // The dynamic shared-memory limit of one instantiation, raised once per
@@ -329,8 +334,7 @@ template <int MAXE, int U>
 int launch_u(const DigestPlan<MAXE> &plan, unsigned grid, void *stream, unsigned long long *out) {
   int e = ensure_stage_attribute<MAXE, U>();
   if (e) return e;
-  digest_kernel<MAXE, U><<<grid, kThreads, launch_smem<U>(), (cudaStream_t)stream>>>(plan, out);
-  return (int)cudaGetLastError();
+  return launch_plan(digest_kernel<MAXE, U>, plan, plan.chained, grid, kThreads, launch_smem<U>(), stream, out);
 }
 
 template <int MAXE>

@@ -26,6 +26,7 @@
 #include "../../include/apc.h"
 #include "apc_device.cuh"
 #include "apc_internal.h"
+#include "apc_launch.cuh"
 
 namespace apc {
 namespace {
@@ -48,6 +49,7 @@ template <int MAXE>
 __global__ void __launch_bounds__(kCountThreads, 1) count_kernel(const __grid_constant__ DigestPlan<MAXE> plan,
                                                          unsigned long long *out) {
   __shared__ unsigned long long s_acc[APC_MAX_SLOTS];
+  if (plan.more) chain_start_next();
   if (threadIdx.x < APC_MAX_SLOTS) s_acc[threadIdx.x] = 0;
   __syncthreads();
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -101,19 +103,20 @@ __global__ void __launch_bounds__(kCountThreads, 1) count_kernel(const __grid_co
   }
   flush(acc, slot, s_acc);
   __syncthreads();
-  if (threadIdx.x < APC_MAX_SLOTS && s_acc[threadIdx.x]) atomicAdd(&out[threadIdx.x], s_acc[threadIdx.x]);
+  if (threadIdx.x < APC_MAX_SLOTS) {
+    chain_wait();
+    if (s_acc[threadIdx.x]) atomicAdd(&out[threadIdx.x], s_acc[threadIdx.x]);
+  }
 }
 
 }  // namespace
 
 int launch_count_small(const DigestPlan<kDigestSmall> &plan, unsigned grid, void *stream, unsigned long long *out) {
-  count_kernel<kDigestSmall><<<grid, kCountThreads, 0, (cudaStream_t)stream>>>(plan, out);
-  return (int)cudaGetLastError();
+  return launch_plan(count_kernel<kDigestSmall>, plan, plan.chained, grid, kCountThreads, 0, stream, out);
 }
 
 int launch_count_large(const DigestPlan<kDigestLarge> &plan, unsigned grid, void *stream, unsigned long long *out) {
-  count_kernel<kDigestLarge><<<grid, kCountThreads, 0, (cudaStream_t)stream>>>(plan, out);
-  return (int)cudaGetLastError();
+  return launch_plan(count_kernel<kDigestLarge>, plan, plan.chained, grid, kCountThreads, 0, stream, out);
 }
 
 int count_blocks_per_sm(bool large, int *out) {

@@ -174,6 +174,15 @@ apc_status device_info(Device *out) {
   return APC_OK;
 }
 
+// The launches of a long table go onto their stream as one chain (launch_plan):
+// a chain of another thread on the same stream must not mix with them.  (A
+// single launch may come in between: it starts nothing early.)
+std::mutex &chain_lock(const void *stream) {
+  static std::mutex locks[64];
+  const uintptr_t s = (uintptr_t)stream;
+  return locks[(s ^ s >> 6 ^ s >> 12) & 63];
+}
+
 // SMs that the persistent kernels leave free (apc_set_reserved_sms).
 std::atomic<int> g_reserved_sms{0};
 
@@ -326,6 +335,8 @@ apc_status run_commit_batches(const std::vector<apc::CommitEntry> &entries, cons
   std::unique_ptr<apc::CommitPlan<MAXE>> plan(new apc::CommitPlan<MAXE>);  // not cleared: the kernel reads what is filled
   commit_scalars(h, plan.get());
   plan->one = 1;
+  std::unique_lock<std::mutex> chain;
+  if (entries.size() > (size_t)MAXE) chain = std::unique_lock<std::mutex>(chain_lock(stream));
   size_t i = 0;
   while (i < entries.size()) {
     const size_t k = std::min(entries.size() - i, (size_t)MAXE);
@@ -340,6 +351,8 @@ apc_status run_commit_batches(const std::vector<apc::CommitEntry> &entries, cons
     plan->tile = tile;
     plan->count = (uint32_t)k;
     plan->total_tiles = tiles;
+    plan->more = i + k < entries.size();
+    plan->chained = i > 0;
     const uint64_t want = std::max<uint64_t>(tiles, k);
     const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(want, grid_cap));
     int e = launch(*plan, layout, zero_grad, grid, stream, out);
@@ -352,10 +365,12 @@ apc_status run_commit_batches(const std::vector<apc::CommitEntry> &entries, cons
 // Entries arrive with the element count of their vector body in tile_begin;
 // tiles_of(body, element size) is the kernel's count of whole tiles in it.
 template <int MAXE, typename Tiles, typename Launch>
-apc_status run_digest_batches(const std::vector<apc::DigestEntry> &entries, unsigned grid_cap, Tiles tiles_of,
-                              Launch launch, const char *what) {
+apc_status run_digest_batches(const std::vector<apc::DigestEntry> &entries, unsigned grid_cap, const void *stream,
+                              Tiles tiles_of, Launch launch, const char *what) {
   std::unique_ptr<apc::DigestPlan<MAXE>> plan(new apc::DigestPlan<MAXE>);
   plan->one = 1;
+  std::unique_lock<std::mutex> chain;
+  if (entries.size() > (size_t)MAXE) chain = std::unique_lock<std::mutex>(chain_lock(stream));
   size_t i = 0;
   while (i < entries.size()) {
     const size_t k = std::min(entries.size() - i, (size_t)MAXE);
@@ -371,6 +386,8 @@ apc_status run_digest_batches(const std::vector<apc::DigestEntry> &entries, unsi
     plan->count = (uint32_t)k;
     plan->total_tiles = tiles;
     plan->tiles32 = tiles32;
+    plan->more = i + k < entries.size();
+    plan->chained = i > 0;
     const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(std::max<uint64_t>(tiles, k), grid_cap));
     int e = launch(*plan, grid);
     if (e) return cuda_fail(e, what);
@@ -465,12 +482,12 @@ apc_status commit_common(int layout, const std::vector<TableRow> &rows, const ap
     return fail(APC_EINVAL, "table buffers or out_digests overlap (a written range meets another range)");
   if ((st = check_device_pointers(ordered, ranges.size(), "out_digests")) != APC_OK) return st;
 
-  int e = (int)cudaMemsetAsync(out_digests, 0, (size_t)nslots * sizeof(uint64_t), (cudaStream_t)stream);
+  unsigned long long *out = reinterpret_cast<unsigned long long *>(out_digests);
+  Device d;
+  if (!entries.empty() && (st = device_info(&d)) != APC_OK) return st;
+  int e = (int)cudaMemsetAsync(out, 0, (size_t)nslots * sizeof(uint64_t), (cudaStream_t)stream);
   if (e) return cuda_fail(e, "cudaMemsetAsync(out_digests)");
   if (entries.empty()) return APC_OK;
-  Device d;
-  if ((st = device_info(&d)) != APC_OK) return st;
-  unsigned long long *out = reinterpret_cast<unsigned long long *>(out_digests);
   if (entries.size() <= (size_t)apc::kCommitSmall)
     return run_commit_batches<apc::kCommitSmall>(entries, h, layout, zero_grad,
                                                  grid_for(UINT64_MAX, d.sms, d.commit_small), stream, out,
@@ -576,12 +593,12 @@ APC_EXPORT apc_status apc_digest(const apc_buffer *bufs, int32_t num_bufs, int32
   std::vector<apc::DigestEntry> entries;
   apc_status st = buffer_entries(bufs, num_bufs, num_slots, out_digests, &entries);
   if (st != APC_OK) return st;
-  int e = (int)cudaMemsetAsync(out_digests, 0, (size_t)num_slots * sizeof(uint64_t), (cudaStream_t)stream);
+  unsigned long long *out = reinterpret_cast<unsigned long long *>(out_digests);
+  Device d;
+  if (!entries.empty() && (st = device_info(&d)) != APC_OK) return st;
+  int e = (int)cudaMemsetAsync(out, 0, (size_t)num_slots * sizeof(uint64_t), (cudaStream_t)stream);
   if (e) return cuda_fail(e, "cudaMemsetAsync(out_digests)");
   if (entries.empty()) return APC_OK;
-  Device d;
-  if ((st = device_info(&d)) != APC_OK) return st;
-  unsigned long long *out = reinterpret_cast<unsigned long long *>(out_digests);
   const bool small = entries.size() <= (size_t)apc::kDigestSmall;
   const unsigned cap = grid_for(UINT64_MAX, d.sms, small ? d.digest_small : d.digest_large);
   // long tiles where every warp of the grid gets several of them in a launch
@@ -594,10 +611,10 @@ APC_EXPORT apc_status apc_digest(const apc_buffer *bufs, int32_t num_bufs, int32
   const auto tiles_of = [u](uint64_t n, uint64_t) { return n / apc::digest_tile(u); };
   if (small)
     return run_digest_batches<apc::kDigestSmall>(
-        entries, cap, tiles_of, [&](const auto &plan, unsigned grid) { return apc::launch_digest_small(plan, u, grid, stream, out); },
+        entries, cap, stream, tiles_of, [&](const auto &plan, unsigned grid) { return apc::launch_digest_small(plan, u, grid, stream, out); },
         "digest kernel launch");
   return run_digest_batches<apc::kDigestLarge>(
-      entries, cap, tiles_of, [&](const auto &plan, unsigned grid) { return apc::launch_digest_large(plan, u, grid, stream, out); },
+      entries, cap, stream, tiles_of, [&](const auto &plan, unsigned grid) { return apc::launch_digest_large(plan, u, grid, stream, out); },
       "digest kernel launch");
 }
 
@@ -607,20 +624,20 @@ APC_EXPORT apc_status apc_count_nonzero(const apc_buffer *bufs, int32_t num_bufs
   std::vector<apc::DigestEntry> entries;
   apc_status st = buffer_entries(bufs, num_bufs, num_slots, out_counts, &entries);
   if (st != APC_OK) return st;
-  int e = (int)cudaMemsetAsync(out_counts, 0, (size_t)num_slots * sizeof(uint64_t), (cudaStream_t)stream);
+  Device d;
+  if (!entries.empty() && (st = device_info(&d)) != APC_OK) return st;
+  unsigned long long *out = reinterpret_cast<unsigned long long *>(out_counts);
+  int e = (int)cudaMemsetAsync(out, 0, (size_t)num_slots * sizeof(uint64_t), (cudaStream_t)stream);
   if (e) return cuda_fail(e, "cudaMemsetAsync(out_counts)");
   if (entries.empty()) return APC_OK;
-  Device d;
-  if ((st = device_info(&d)) != APC_OK) return st;
-  unsigned long long *out = reinterpret_cast<unsigned long long *>(out_counts);
   const auto tiles_of = [](uint64_t n, uint64_t es) { return n * es / apc::kCountTileBytes; };
   if (entries.size() <= (size_t)apc::kDigestSmall)
     return run_digest_batches<apc::kDigestSmall>(
-        entries, grid_for(UINT64_MAX, d.sms, d.count_small), tiles_of,
+        entries, grid_for(UINT64_MAX, d.sms, d.count_small), stream, tiles_of,
         [&](const auto &plan, unsigned grid) { return apc::launch_count_small(plan, grid, stream, out); },
         "count kernel launch");
   return run_digest_batches<apc::kDigestLarge>(
-      entries, grid_for(UINT64_MAX, d.sms, d.count_large), tiles_of,
+      entries, grid_for(UINT64_MAX, d.sms, d.count_large), stream, tiles_of,
       [&](const auto &plan, unsigned grid) { return apc::launch_count_large(plan, grid, stream, out); },
       "count kernel launch");
 }

@@ -315,3 +315,52 @@ def test_upload_every_relative_offset(ctas):
     flat = torch.full_like(dst, 0xEE)            # and from device memory
     apc.upload([apc.Segment(flat[d:d + n], dst[d:d + n]) for _, d, n in segs], ctas)
     assert np.array_equal(flat.cpu().numpy(), ref)
+
+
+def test_long_tables_chained_and_captured():
+    """A table of several launches, committed and verified back to back on one
+    stream, eagerly and as a replayed graph: each verification sees the whole
+    commit before it, each commit the whole state before it."""
+    rng = np.random.default_rng(41)
+    sizes = rng.integers(1, 3000, size=1000)
+    goffs = np.concatenate([[0], np.cumsum(sizes)[:-1]]) + 5
+    at = np.concatenate([[0], np.cumsum((sizes + 15) // 16 * 16)])
+    flat = state_words(int(at[-1]), 5, 4, "f32")
+    start = {k: dev_words(flat[k]) for k in "pmvg"}
+    d = {k: t.clone() for k, t in start.items()}
+    d["w"] = torch.zeros_like(d["g"])
+    cut = lambda k, i: d[k][at[i]:at[i] + sizes[i]]
+    e = [apc.TensorEntry(*(cut(k, i) for k in "pmvgw"), int(goffs[i])) for i in range(1000)]
+    table = apc.prepare_table(e)
+    bufs = apc.prepare_buffers([b for t in e for b in apc.state_buffers(t.p, t.m, t.v, t.w, t.global_offset)])
+    outs = [torch.zeros(4, dtype=torch.int64, device="cuda") for _ in range(8)]
+    s = torch.cuda.Stream()
+
+    def three_steps():
+        for j in range(4):
+            apc.commit_step(table, 4, stream=s, out=outs[2 * j])
+            apc.digest(bufs, 4, stream=s, out=outs[2 * j + 1])
+
+    three_steps()
+    torch.cuda.synchronize()
+    eager = [apc.digests_to_host(o) for o in outs]
+    for k in "pmv":
+        d[k].copy_(start[k])
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(s), torch.cuda.graph(graph, stream=s):
+        three_steps()
+    for o in outs:
+        o.zero_()
+    torch.cuda.synchronize()
+    graph.replay()
+    torch.cuda.synchronize()
+    replayed = [apc.digests_to_host(o) for o in outs]
+    h8 = oracle.resolve_hparams(oracle.DEFAULT_HP, 4)
+    ref = [dict(p=flat["p"][a:a + n].view(np.float32).copy(), m=flat["m"][a:a + n].view(np.float32).copy(),
+                v=flat["v"][a:a + n].view(np.float32).copy(), g=flat["g"][a:a + n], goff=int(o))
+           for a, n, o in zip(at, sizes, goffs)]
+    for j in range(4):
+        _, want = oracle.commit_table(ref, h8)
+        assert eager[2 * j] == want and eager[2 * j + 1] == want, j
+        assert replayed[2 * j] == want and replayed[2 * j + 1] == want, j
