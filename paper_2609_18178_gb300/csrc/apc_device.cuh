@@ -170,9 +170,11 @@ __device__ __forceinline__ void adamw_group(float (&p)[N], float (&m)[N], float 
 //  * MulWide: three multiply-adds, lo*clo widened, then lo*chi and hi*clo
 //    added into the high word.  Fewest instructions; the commit kernel,
 //    which is bound by instruction issue, runs 2.7% faster with it.
-//  * MulCompiler: the compiler's own 64-bit multiply.  The verification
-//    pass, which is bound by the integer ALU rather than by issue, runs 3.3%
-//    faster with it.
+//  * MulCompiler: the compiler's own 64-bit multiply, one instruction more and
+//    a shorter chain.  The verification pass's fp32 terms take MulWide first
+//    and this one second: 453 M elements of fp32 state in 1,411 us, against
+//    1,425 with this one twice, 1,419 with MulWide twice, 1,414 the other way
+//    round.
 struct MulWide {
   template <uint32_t CLO, uint32_t CHI>
   __device__ __forceinline__ static uint64_t mul(uint64_t z) {
@@ -214,7 +216,7 @@ struct MulCompiler {
 // high word.  Callers that know them for a whole run of terms pass them as
 // `hi_top` (see digest_term's four-argument form); otherwise they are
 // computed here.
-template <uint32_t K, class Mul>
+template <uint32_t K, class Mul1, class Mul2>
 __device__ __forceinline__ uint64_t digest_term_core(uint32_t gidx, uint32_t bits, uint32_t one, bool have_top,
                                                      uint32_t hi_top) {
   uint32_t lo, hi;
@@ -225,14 +227,14 @@ __device__ __forceinline__ uint64_t digest_term_core(uint32_t gidx, uint32_t bit
   const uint32_t l1 = lo ^ __funnelshift_r(lo, hi, 30);
   const uint32_t h1 = hi ^ (have_top ? hi_top : hi >> 30);
   uint64_t z = ((uint64_t)h1 << 32) | l1;
-  z = Mul::template mul<0x1CE4E5B9u, 0xBF58476Du>(z);
-  z = Mul::template mul<0x133111EBu, 0x94D049BBu>(z ^ (z >> 27));
+  z = Mul1::template mul<0x1CE4E5B9u, 0xBF58476Du>(z);
+  z = Mul2::template mul<0x133111EBu, 0x94D049BBu>(z ^ (z >> 27));
   return z ^ (z >> 31);
 }
 
-template <uint32_t K = 0, class Mul = MulWide>
+template <uint32_t K = 0, class Mul1 = MulWide, class Mul2 = MulWide>
 __device__ __forceinline__ uint64_t digest_term(uint32_t gidx, uint32_t bits, uint32_t one) {
-  return digest_term_core<K, Mul>(gidx, bits, one, false, 0);
+  return digest_term_core<K, Mul1, Mul2>(gidx, bits, one, false, 0);
 }
 
 // The same term with hi >> 30 supplied: hi_top must equal the top two bits
@@ -240,9 +242,9 @@ __device__ __forceinline__ uint64_t digest_term(uint32_t gidx, uint32_t bits, ui
 // [G0, G0 + R), every incremented high word lies in [B, B + R] with
 // B = G0 + 0x9E3779B9 (the carry adds at most 1); when B and B + R have the
 // same top two bits (top_bits_shared), those bits are B >> 30 for all of them.
-template <uint32_t K = 0, class Mul = MulWide>
+template <uint32_t K = 0, class Mul1 = MulWide, class Mul2 = MulWide>
 __device__ __forceinline__ uint64_t digest_term(uint32_t gidx, uint32_t bits, uint32_t one, uint32_t hi_top) {
-  return digest_term_core<K, Mul>(gidx, bits, one, true, hi_top);
+  return digest_term_core<K, Mul1, Mul2>(gidx, bits, one, true, hi_top);
 }
 
 // splitmix64 terms of 16-bit words (bits < 2^16).  Their low key half plus

@@ -63,11 +63,10 @@ struct Shape {
   static constexpr uint32_t kKeySpan32 = (kGroups32 - 1) * kSpan32 + 4, kKeySpan16 = (kGroups16 - 1) * kSpan16 + 8;
 };
 
-// One digest term of this pass.  The pass is bound by the integer ALU, not
-// by issue, and runs faster with the compiler's own 64-bit multiply.
+// One digest term of this pass, in the fp32 terms' mix of multiplies.
 template <uint32_t K>
 __device__ __forceinline__ uint64_t term(uint32_t gidx, uint32_t bits, uint32_t one) {
-  return digest_term<K, MulCompiler>(gidx, bits, one);
+  return digest_term<K, MulWide, MulCompiler>(gidx, bits, one);
 }
 
 // The same with SHARED: the caller has checked that all of a thread's terms
@@ -76,8 +75,8 @@ __device__ __forceinline__ uint64_t term(uint32_t gidx, uint32_t bits, uint32_t 
 // no term computes hi >> 30 itself.
 template <uint32_t K, bool SHARED>
 __device__ __forceinline__ uint64_t vterm(uint32_t gidx, uint32_t bits, uint32_t one, uint32_t top) {
-  if constexpr (SHARED) return digest_term<K, MulCompiler>(gidx, bits, one, top);
-  else return digest_term<K, MulCompiler>(gidx, bits, one);
+  if constexpr (SHARED) return digest_term<K, MulWide, MulCompiler>(gidx, bits, one, top);
+  else return digest_term<K, MulWide, MulCompiler>(gidx, bits, one);
 }
 
 // A thread's terms of one fp32 tile.
