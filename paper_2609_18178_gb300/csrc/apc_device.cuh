@@ -250,25 +250,20 @@ __device__ __forceinline__ uint64_t digest_term(uint32_t gidx, uint32_t bits, ui
 // splitmix64 terms of 16-bit words (bits < 2^16).  Their low key half plus
 // 0x7F4A7C15 never carries and always has top bits 01, so after the
 // increment lo = bits + 0x7F4A7C15, hi = gidx + 0x9E3779B9 + K, and the
-// first xor-shift's low word is lo ^ ((hi << 2) | 1) = lo ^ (4 * hi + 1), with
-// the key's part on the FMA pipe (multiply-adds by `one`); `top` is hi >> 30,
-// shared by the caller (digest_term's hi_top rule).
+// first xor-shift's low word is lo ^ ((hi << 2) | 1) = lo ^ (4 * hi + 1); `top`
+// is hi >> 30, shared by the caller (digest_term's hi_top rule).
 //
 // Term of half HALF (0 low, 1 high) of two packed words.  The half is
 // taken and the increment added by one two-way dot product (dp2a with a unit
-// vector) in place of a mask or shift and a multiply-add.  The commit kernel
-// takes its 16-bit words this way (152 M elements of fp32 state 677 to 667 us,
-// 453 M with zeroed gradients 2,071 to 2,050, 1.81 G of bf16 state 6,067 to
-// 6,042).  The keyed form below saves instructions there too, but spills at
-// the bf16 layout's 72 registers and was no faster.
+// vector) in place of a mask or shift and an add.  The key's part is left to
+// the compiler, which places it on either pipe and shares it between the three
+// words of a bf16-state element (1.81 G elements in 5,693 us; 5,733 with
+// explicit multiply-adds for it).  The keyed form below saves more
+// instructions but spills at the bf16 layout's 72 registers and was no faster.
 template <uint32_t K, int HALF>
 __device__ __forceinline__ uint64_t digest_term_half(uint32_t gidx, uint32_t pair, uint32_t one, uint32_t top) {
   const uint32_t lo = __dp2a_lo(pair, HALF ? 0x0100u : 0x0001u, 0x7F4A7C15u);
-  uint32_t hi, m4;
-  asm("mad.lo.u32 %0, %2, %4, %3;\n\t"
-      "mad.lo.u32 %1, %0, 4, %2;"
-      : "=r"(hi), "=r"(m4)
-      : "r"(one), "r"(gidx), "n"(0x9E3779B9u + K));
+  const uint32_t hi = gidx + (0x9E3779B9u + K), m4 = 4 * hi + 1;
   const uint32_t l1 = lo ^ m4, h1 = hi ^ top;
   uint64_t z = ((uint64_t)h1 << 32) | l1;
   z = MulWide::template mul<0x1CE4E5B9u, 0xBF58476Du>(z);
