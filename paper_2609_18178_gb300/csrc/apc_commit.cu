@@ -689,51 +689,42 @@ int launch_l(const CommitPlan<MAXE> &plan, bool zero_grad, unsigned grid, void *
                    : launch_t<L, MAXE, false, false>(plan, grid, stream, out);
 }
 
-template <int MAXE>
-int launch(const CommitPlan<MAXE> &plan, int layout, bool zero_grad, unsigned grid, void *stream,
-           unsigned long long *out) {
-  return layout == kLayoutBF16 ? launch_l<BF16State>(plan, zero_grad, grid, stream, out)
-                               : launch_l<F32State>(plan, zero_grad, grid, stream, out);
-}
-
 template <class L, int MAXE, bool MIS>
-int blocks_m(int *out) {
+int blocks_m(int *fewest) {
+  int n = 0;
   int e = ensure_smem_attribute<L, MAXE, false, MIS>();
   if (e) return e;
-  return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, commit_kernel<L, MAXE, false, MIS>, L::kThreads,
-                                                            smem_bytes<L, MIS>());
+  e = (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, commit_kernel<L, MAXE, false, MIS>, L::kThreads,
+                                                         smem_bytes<L, MIS>());
+  if (n < *fewest) *fewest = n;
+  return e;
 }
 
-template <class L, int MAXE>
-int blocks_per_sm(int *out) {
-  int a = 0, b = 0;
-  int e = blocks_m<L, MAXE, false>(&a);
-  if (e || (e = blocks_m<L, MAXE, true>(&b))) return e;
-  *out = a < b ? a : b;
-  return 0;
+template <int MAXE>
+int blocks_n(int *fewest) {
+  int e = blocks_m<F32State, MAXE, false>(fewest);
+  if (!e) e = blocks_m<F32State, MAXE, true>(fewest);
+  if (!e) e = blocks_m<BF16State, MAXE, false>(fewest);
+  return e ? e : blocks_m<BF16State, MAXE, true>(fewest);
 }
 
 }  // namespace
 
-int launch_commit_small(const CommitPlan<kCommitSmall> &plan, int layout, bool zero_grad, unsigned grid,
-                        void *stream, unsigned long long *out) {
-  return launch(plan, layout, zero_grad, grid, stream, out);
+template <int MAXE>
+int launch_commit(const CommitPlan<MAXE> &plan, int layout, bool zero_grad, unsigned grid, void *stream,
+                  unsigned long long *out) {
+  return layout == kLayoutBF16 ? launch_l<BF16State>(plan, zero_grad, grid, stream, out)
+                               : launch_l<F32State>(plan, zero_grad, grid, stream, out);
 }
+template int launch_commit(const CommitPlan<kCommitSmall> &, int, bool, unsigned, void *, unsigned long long *);
+template int launch_commit(const CommitPlan<kCommitMid> &, int, bool, unsigned, void *, unsigned long long *);
+template int launch_commit(const CommitPlan<kCommitLarge> &, int, bool, unsigned, void *, unsigned long long *);
 
-int launch_commit_large(const CommitPlan<kCommitLarge> &plan, int layout, bool zero_grad, unsigned grid,
-                        void *stream, unsigned long long *out) {
-  return launch(plan, layout, zero_grad, grid, stream, out);
-}
-
-int commit_blocks_per_sm(bool large, int *out) {
-  // one grid size serves all instantiations: the smaller of their residencies
-  int f = 0, b = 0;
-  int e = large ? blocks_per_sm<F32State, kCommitLarge>(&f) : blocks_per_sm<F32State, kCommitSmall>(&f);
-  if (e) return e;
-  e = large ? blocks_per_sm<BF16State, kCommitLarge>(&b) : blocks_per_sm<BF16State, kCommitSmall>(&b);
-  if (e) return e;
-  *out = f < b ? f : b;
-  return 0;
+int commit_blocks_per_sm(int *out) {
+  *out = 1 << 20;
+  int e = blocks_n<kCommitSmall>(out);
+  if (!e) e = blocks_n<kCommitMid>(out);
+  return e ? e : blocks_n<kCommitLarge>(out);
 }
 
 int launch_wait_timeout(uint64_t limit_ns, void *stream) {

@@ -336,41 +336,38 @@ int launch_u(const DigestPlan<MAXE> &plan, unsigned grid, void *stream, unsigned
   return launch_plan(digest_kernel<MAXE, U>, plan, plan.chained, grid, kThreads, launch_smem<U>(), stream, out);
 }
 
-template <int MAXE>
-int launch_t(const DigestPlan<MAXE> &plan, int u, unsigned grid, void *stream, unsigned long long *out) {
-  return u == kDigestLong ? launch_u<MAXE, kDigestLong>(plan, grid, stream, out)
-                          : launch_u<MAXE, kDigestShort>(plan, grid, stream, out);
-}
-
 template <int MAXE, int U>
-int blocks_u(int *out) {
+int blocks_u(int *fewest) {
+  int n = 0;
   int e = ensure_stage_attribute<MAXE, U>();
   if (e) return e;
-  return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, digest_kernel<MAXE, U>, kThreads, launch_smem<U>());
+  e = (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, digest_kernel<MAXE, U>, kThreads, launch_smem<U>());
+  if (n < *fewest) *fewest = n;
+  return e;
 }
 
-// One grid size serves both tile lengths: the smaller of their residencies.
 template <int MAXE>
-int blocks_t(int *out) {
-  int a = 0, b = 0;
-  int e = blocks_u<MAXE, kDigestShort>(&a);
-  if (e || (e = blocks_u<MAXE, kDigestLong>(&b))) return e;
-  *out = a < b ? a : b;
-  return 0;
+int blocks_n(int *fewest) {
+  const int e = blocks_u<MAXE, kDigestShort>(fewest);
+  return e ? e : blocks_u<MAXE, kDigestLong>(fewest);
 }
 
 }  // namespace
 
-int launch_digest_small(const DigestPlan<kDigestSmall> &plan, int u, unsigned grid, void *stream,
-                        unsigned long long *out) {
-  return launch_t<kDigestSmall>(plan, u, grid, stream, out);
+template <int MAXE>
+int launch_digest(const DigestPlan<MAXE> &plan, int u, unsigned grid, void *stream, unsigned long long *out) {
+  return u == kDigestLong ? launch_u<MAXE, kDigestLong>(plan, grid, stream, out)
+                          : launch_u<MAXE, kDigestShort>(plan, grid, stream, out);
 }
+template int launch_digest(const DigestPlan<kDigestSmall> &, int, unsigned, void *, unsigned long long *);
+template int launch_digest(const DigestPlan<kDigestMid> &, int, unsigned, void *, unsigned long long *);
+template int launch_digest(const DigestPlan<kDigestLarge> &, int, unsigned, void *, unsigned long long *);
 
-int launch_digest_large(const DigestPlan<kDigestLarge> &plan, int u, unsigned grid, void *stream,
-                        unsigned long long *out) {
-  return launch_t<kDigestLarge>(plan, u, grid, stream, out);
+int digest_blocks_per_sm(int *out) {
+  *out = 1 << 20;
+  int e = blocks_n<kDigestSmall>(out);
+  if (!e) e = blocks_n<kDigestMid>(out);
+  return e ? e : blocks_n<kDigestLarge>(out);
 }
-
-int digest_blocks_per_sm(bool large, int *out) { return large ? blocks_t<kDigestLarge>(out) : blocks_t<kDigestSmall>(out); }
 
 }  // namespace apc

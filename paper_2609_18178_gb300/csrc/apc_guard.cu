@@ -109,20 +109,29 @@ __global__ void __launch_bounds__(kCountThreads, 1) count_kernel(const __grid_co
   }
 }
 
+template <int MAXE>
+int blocks_n(int *fewest) {
+  int n = 0;
+  const int e = (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, count_kernel<MAXE>, kCountThreads, 0);
+  if (n < *fewest) *fewest = n;
+  return e;
+}
+
 }  // namespace
 
-int launch_count_small(const DigestPlan<kDigestSmall> &plan, unsigned grid, void *stream, unsigned long long *out) {
-  return launch_plan(count_kernel<kDigestSmall>, plan, plan.chained, grid, kCountThreads, 0, stream, out);
+template <int MAXE>
+int launch_count(const DigestPlan<MAXE> &plan, unsigned grid, void *stream, unsigned long long *out) {
+  return launch_plan(count_kernel<MAXE>, plan, plan.chained, grid, kCountThreads, 0, stream, out);
 }
+template int launch_count(const DigestPlan<kDigestSmall> &, unsigned, void *, unsigned long long *);
+template int launch_count(const DigestPlan<kDigestMid> &, unsigned, void *, unsigned long long *);
+template int launch_count(const DigestPlan<kDigestLarge> &, unsigned, void *, unsigned long long *);
 
-int launch_count_large(const DigestPlan<kDigestLarge> &plan, unsigned grid, void *stream, unsigned long long *out) {
-  return launch_plan(count_kernel<kDigestLarge>, plan, plan.chained, grid, kCountThreads, 0, stream, out);
-}
-
-int count_blocks_per_sm(bool large, int *out) {
-  cudaError_t e = large ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, count_kernel<kDigestLarge>, kCountThreads, 0)
-                        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, count_kernel<kDigestSmall>, kCountThreads, 0);
-  return (int)e;
+int count_blocks_per_sm(int *out) {
+  *out = 1 << 20;
+  int e = blocks_n<kDigestSmall>(out);
+  if (!e) e = blocks_n<kDigestMid>(out);
+  return e ? e : blocks_n<kDigestLarge>(out);
 }
 
 }  // namespace apc

@@ -139,8 +139,9 @@ struct CommitPlan {
   CommitEntry e[MAXE];
 };
 
-constexpr int kCommitSmall = 16;
-constexpr int kCommitLarge = 440;
+// Plans of three sizes: a launch copies its whole parameter block, which takes
+// 1 to 1.5 us more for 32 KB than for 7 (with_plan).
+constexpr int kCommitSmall = 16, kCommitMid = 96, kCommitLarge = 440;
 static_assert(sizeof(CommitEntry) == 72, "entry layout");
 static_assert(sizeof(CommitPlan<kCommitLarge>) <= 32764, "kernel parameter limit");
 
@@ -218,8 +219,7 @@ struct DigestPlan {
   DigestEntry e[MAXE];
 };
 
-constexpr int kDigestSmall = 16;
-constexpr int kDigestLarge = 1000;
+constexpr int kDigestSmall = 16, kDigestMid = 200, kDigestLarge = 1000;
 static_assert(sizeof(DigestEntry) == 32, "entry layout");
 static_assert(sizeof(DigestPlan<kDigestLarge>) <= 32764, "kernel parameter limit");
 
@@ -264,26 +264,23 @@ static_assert(sizeof(UploadPlan<kUploadMax>) <= 32764, "kernel parameter limit")
 // Upload kernel (apc_upload.cu): the plan's segments, on `grid` CTAs.
 int launch_upload(const UploadPlan<kUploadMax> &plan, unsigned grid, void *stream);
 
-// Launch wrappers (apc_commit.cu, apc_digest.cu).  They return a cudaError_t
-// value and launch on `stream` with `grid` CTAs.
-int launch_commit_small(const CommitPlan<kCommitSmall> &plan, int layout, bool zero_grad, unsigned grid,
-                        void *stream, unsigned long long *out);
-int launch_commit_large(const CommitPlan<kCommitLarge> &plan, int layout, bool zero_grad, unsigned grid,
-                        void *stream, unsigned long long *out);
-int launch_digest_small(const DigestPlan<kDigestSmall> &plan, int u, unsigned grid, void *stream,
-                        unsigned long long *out);
-int launch_digest_large(const DigestPlan<kDigestLarge> &plan, int u, unsigned grid, void *stream,
-                        unsigned long long *out);
+// Launch wrappers (apc_commit.cu, apc_digest.cu, apc_guard.cu), instantiated for
+// the plan sizes above.  They return a cudaError_t value and launch on `stream`
+// with `grid` CTAs; u: the digest kernel's vectors per lane per tile.
+template <int MAXE>
+int launch_commit(const CommitPlan<MAXE> &plan, int layout, bool zero_grad, unsigned grid, void *stream,
+                  unsigned long long *out);
+template <int MAXE>
+int launch_digest(const DigestPlan<MAXE> &plan, int u, unsigned grid, void *stream, unsigned long long *out);
+// Per-slot counts of nonzero words over the same buffer plans as the digest.
+template <int MAXE>
+int launch_count(const DigestPlan<MAXE> &plan, unsigned grid, void *stream, unsigned long long *out);
 
-// Resident CTAs per SM of each kernel (cudaOccupancyMaxActiveBlocksPerMultiprocessor).
-int commit_blocks_per_sm(bool large, int *out);
-int digest_blocks_per_sm(bool large, int *out);
-
-// Count kernel (apc_guard.cu): per-slot counts of nonzero words over the
-// same buffer plans as the digest.
-int launch_count_small(const DigestPlan<kDigestSmall> &plan, unsigned grid, void *stream, unsigned long long *out);
-int launch_count_large(const DigestPlan<kDigestLarge> &plan, unsigned grid, void *stream, unsigned long long *out);
-int count_blocks_per_sm(bool large, int *out);
+// Resident CTAs per SM of each kernel (cudaOccupancyMaxActiveBlocksPerMultiprocessor),
+// the fewest over its instantiations.
+int commit_blocks_per_sm(int *out);
+int digest_blocks_per_sm(int *out);
+int count_blocks_per_sm(int *out);
 
 // Device status word of the kernels of one translation unit on the current
 // device: nonzero after a bounded wait gave up.  read_* copies it to the host
