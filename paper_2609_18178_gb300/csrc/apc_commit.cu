@@ -31,20 +31,21 @@
 //    the global stores are contiguous across the warp), release the
 //    stage to the producer, then apply AdamW, store the results with
 //    streaming stores, and fold the digest terms into 64-bit registers.
-//  * Entries whose buffers are not mutually 16-byte aligned (a packed flat
-//    shard of odd-sized tensors beside gradients and copies with boundaries of
-//    their own) run through the same ring: the producer copies, for each
-//    buffer, the 16-byte blocks that hold the tile, and the consumers read
-//    the words at the buffers' own offsets, lane-consecutive, and store them
-//    one by one.  That keeps whole tiles in flight where element loads straight
-//    from global memory kept one element per thread: 60 M elements in 291 odd
-//    entries take 386 us (606 before, 247 at the copy rate).  Tables without
-//    such an entry run an instantiation without this code (MIS = false).
-//  * What lies outside the tiles (fewer than 8 elements at each end of an
-//    aligned entry, at most 8 and 15 of a misaligned one, whole entries under
-//    32 elements of the latter) is done straight from global memory by the
-//    producer warp once it has issued its copies, so that it costs the
-//    consumers nothing.
+//  * Entries whose buffers are not mutually 16-byte aligned run through the same
+//    ring.  The usual case is a packed flat shard of odd-sized tensors, p, m and
+//    v alike, beside gradients and copies with boundaries of their own: there
+//    p, m and v keep their vectors, the producer copies the 16-byte blocks that
+//    hold the tile's gradient, and the consumers read its words, and store the
+//    copy's, at their own offsets.  Where p, m and v are at odds too, all four
+//    are copied in blocks and every word is read and stored by itself,
+//    lane-consecutive.  60 M elements in 291 odd entries take 281 us, 320
+//    with every word by itself, 606 with element loads straight from global
+//    memory (247 at the copy rate).  Tables without such an entry run an
+//    instantiation without this code (MIS = false).
+//  * What lies outside the tiles (fewer than 8 elements at each end of an aligned
+//    entry, at most 15 of another, whole entries under 32 elements of the latter)
+//    is done straight from global memory by the producer warp once it has issued
+//    its copies, so that it costs the consumers nothing.
 //  * At exit the CTA sums each digest (warp shuffles, shared memory) and adds
 //    it into the caller's output with one 64-bit atomic; addition mod 2^64 is
 //    order-free, so digests do not depend on grid size or table split.
@@ -107,16 +108,28 @@ struct Dst {
 // makes it visible to them): the addresses of the tile's first element in
 // p, m, v, w and g, its element count and its first digest index.  The
 // consumers then spend no instructions locating the tile in the chunk table.
-// A misaligned tile's cnt also holds kMisTile and, from bit 16 on, four bits
-// each: the byte offsets of its first element in the staged blocks of p, m, v
-// and g.
+// Where the entry's buffers are not mutually aligned, cnt also holds, from bit 16
+// on, four bits each: the byte offsets of the tile's first element in the
+// staged blocks of p, m, v and g; and kMisTile, or kHalfTile if only the
+// gradient and the copy are at odds with p, m and v.
 struct __align__(16) StageDesc {
   uint8_t *p, *m, *v;
   uint16_t *w, *g;
   uint32_t cnt, G;
 };
-constexpr uint32_t kMisTile = 1u << 15;
-static_assert(kCommitTile < kMisTile && kCommitTileBF16 < kMisTile, "a tile's count and kMisTile share a word");
+constexpr uint32_t kMisTile = 1u << 15, kHalfTile = 1u << 14, kCntMask = kHalfTile - 1;
+static_assert(kCommitTile <= kCntMask && kCommitTileBF16 <= kCntMask, "a tile's count and its flags share a word");
+
+// Four 16-bit words at any 2-byte address.
+__device__ __forceinline__ uint2 words4(const uint16_t *q) {
+  return make_uint2((uint32_t)q[0] | (uint32_t)q[1] << 16, (uint32_t)q[2] | (uint32_t)q[3] << 16);
+}
+__device__ __forceinline__ void store_words4(uint16_t *q, uint2 x) {
+  __stcs(q, (uint16_t)x.x);
+  __stcs(q + 1, (uint16_t)(x.x >> 16));
+  __stcs(q + 2, (uint16_t)x.y);
+  __stcs(q + 3, (uint16_t)(x.y >> 16));
+}
 static_assert(sizeof(StageDesc) == 48, "three 16-byte shared-memory loads");
 
 // A commit digest term.  With SHARED the caller has established that the
@@ -155,13 +168,15 @@ struct F32State {
     uint2 g;
   };
 
-  // PAD: bytes between the stage's regions (16 where misaligned tiles may come).
+  // PAD: bytes between the stage's regions (16 where misaligned tiles may come);
+  // half: the gradient begins `goff` bytes into its region.
   template <uint32_t PAD>
-  __device__ static void load(const uint8_t *st, uint32_t e, Regs &r) {
+  __device__ static void load(const uint8_t *st, uint32_t e, bool half, uint32_t goff, Regs &r) {
     r.p = *reinterpret_cast<const float4 *>(st + 4 * e);
     r.m = *reinterpret_cast<const float4 *>(st + 4 * (kTile + e) + PAD);
     r.v = *reinterpret_cast<const float4 *>(st + 4 * (2 * kTile + e) + 2 * PAD);
-    r.g = *reinterpret_cast<const uint2 *>(st + 12 * kTile + 2 * e + 3 * PAD);
+    const uint8_t *g = st + 12 * kTile + 2 * e + 3 * PAD;
+    r.g = PAD && half ? words4(reinterpret_cast<const uint16_t *>(g + goff)) : *reinterpret_cast<const uint2 *>(g);
   }
 
   // Where a misaligned tile's elements sit in its stage.
@@ -216,8 +231,8 @@ struct F32State {
 
   // Four consecutive elements at the compile-time element offset OFF from
   // the thread's output addresses, whose first element has digest index G.
-  template <uint32_t OFF, bool ZERO>
-  __device__ static void compute_store(const Dst &d, uint32_t G, const Regs &r, const Scalars &s, Acc &a) {
+  template <uint32_t OFF, bool ZERO, bool MIS>
+  __device__ static void compute_store(const Dst &d, uint32_t G, const Regs &r, bool half, const Scalars &s, Acc &a) {
     constexpr uint32_t off = OFF;
     float p[4] = {r.p.x, r.p.y, r.p.z, r.p.w};
     float m[4] = {r.m.x, r.m.y, r.m.z, r.m.w};
@@ -236,7 +251,8 @@ struct F32State {
     __stcs(reinterpret_cast<float4 *>(static_cast<float *>(d.m) + off), make_float4(m[0], m[1], m[2], m[3]));
     __stcs(reinterpret_cast<float4 *>(static_cast<float *>(d.v) + off), make_float4(v[0], v[1], v[2], v[3]));
     const uint32_t w01 = pack_bf16x2(p[0], p[1]), w23 = pack_bf16x2(p[2], p[3]);
-    __stcs(reinterpret_cast<uint2 *>(d.w + off), make_uint2(w01, w23));
+    if (MIS && half) store_words4(d.w + off, make_uint2(w01, w23));
+    else __stcs(reinterpret_cast<uint2 *>(d.w + off), make_uint2(w01, w23));
     // the group's keys are G + OFF .. G + OFF + 3
     const uint32_t B = G + (0x9E3779B9u + OFF);
     const uint32_t pb[4] = {__float_as_uint(p[0]), __float_as_uint(p[1]), __float_as_uint(p[2]), __float_as_uint(p[3])};
@@ -296,11 +312,12 @@ struct BF16State {
   };
 
   template <uint32_t PAD>
-  __device__ static void load(const uint8_t *st, uint32_t e, Regs &r) {
+  __device__ static void load(const uint8_t *st, uint32_t e, bool half, uint32_t goff, Regs &r) {
     r.p = *reinterpret_cast<const uint2 *>(st + 2 * e);
     r.m = *reinterpret_cast<const uint2 *>(st + 2 * (kTile + e) + PAD);
     r.v = *reinterpret_cast<const uint2 *>(st + 2 * (2 * kTile + e) + 2 * PAD);
-    r.g = *reinterpret_cast<const uint2 *>(st + 6 * kTile + 2 * e + 3 * PAD);
+    const uint8_t *g = st + 6 * kTile + 2 * e + 3 * PAD;
+    r.g = PAD && half ? words4(reinterpret_cast<const uint16_t *>(g + goff)) : *reinterpret_cast<const uint2 *>(g);
   }
 
   struct Mis {
@@ -348,8 +365,8 @@ struct BF16State {
     if (ZERO) __stcs(sd.g + e, (uint16_t)0);
   }
 
-  template <uint32_t OFF, bool ZERO>
-  __device__ static void compute_store(const Dst &d, uint32_t G, const Regs &r, const Scalars &s, Acc &a) {
+  template <uint32_t OFF, bool ZERO, bool MIS>
+  __device__ static void compute_store(const Dst &d, uint32_t G, const Regs &r, bool half, const Scalars &s, Acc &a) {
     constexpr uint32_t off = OFF;
     const uint32_t pw[4] = {r.p.x & 0xFFFFu, r.p.x >> 16, r.p.y & 0xFFFFu, r.p.y >> 16};
     const uint32_t mw[4] = {r.m.x & 0xFFFFu, r.m.x >> 16, r.m.y & 0xFFFFu, r.m.y >> 16};
@@ -405,15 +422,18 @@ struct BF16State {
 // offset K * 4 * L::kConsumers from the thread's output addresses, which
 // the stores carry as immediates and the digest terms fold into their
 // increment.
-template <class L, bool ZERO, int K>
-__device__ __forceinline__ void store_groups(const Dst &d, uint32_t G1, const typename L::Regs *r, const bool *ok,
+template <class L, bool ZERO, bool MIS, int K>
+__device__ __forceinline__ void store_groups(const Dst &d, uint32_t G1, const typename L::Regs *r, const bool *ok, bool half,
                                              const Scalars &s, Acc &a) {
   constexpr uint32_t off = (uint32_t)(K * L::kConsumers) * 4;
   if (ok[K]) {
-    if (ZERO) __stcs(reinterpret_cast<uint2 *>(d.g + off), make_uint2(0u, 0u));
-    L::template compute_store<off, ZERO>(d, G1, r[K], s, a);
+    if (ZERO) {
+      if (MIS && half) store_words4(d.g + off, make_uint2(0u, 0u));
+      else __stcs(reinterpret_cast<uint2 *>(d.g + off), make_uint2(0u, 0u));
+    }
+    L::template compute_store<off, ZERO, MIS>(d, G1, r[K], half, s, a);
   }
-  if constexpr (K + 1 < L::kGroups) store_groups<L, ZERO, K + 1>(d, G1, r, ok, s, a);
+  if constexpr (K + 1 < L::kGroups) store_groups<L, ZERO, MIS, K + 1>(d, G1, r, ok, half, s, a);
 }
 
 // The stage's four regions; with MIS each has 16 bytes more, for the blocks
@@ -436,21 +456,6 @@ __device__ __forceinline__ void copy_blocks(uint8_t *dst, const uint8_t *src, ui
                                             uint64_t policy) {
   const uint32_t off = (uint32_t)((uintptr_t)src & 15);
   bulk_g2s(dst, src - off, (off + bytes + 15) & ~15u, bar, policy);
-}
-
-// The entry that holds `tile` (the last that begins at or before it; entries
-// without tiles begin where the next one does), by bisection: a walk from the
-// first entry took 440 dependent constant loads in a CTA near a full table's
-// end.  The producer then walks on from there.
-template <int MAXE>
-__device__ __forceinline__ uint32_t first_entry(const CommitPlan<MAXE> &plan, uint64_t tile) {
-  uint32_t lo = 0, hi = plan.count;
-  while (hi - lo > 1) {
-    const uint32_t mid = (lo + hi) >> 1;
-    if (plan.e[mid].tile_begin <= tile) lo = mid;
-    else hi = mid;
-  }
-  return lo;
 }
 
 template <int MAXE>
@@ -507,7 +512,7 @@ __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
     if (lane == 0) {
       const uint64_t policy = l2_evict_first();
       const TileWalk w = tile_walk(plan.total_tiles);
-      uint32_t cur = w.t0 < w.t1 ? first_entry(plan, w.t0) : 0;
+      uint32_t cur = w.t0 < w.t1 ? entry_of(plan, 0, w.t0) : 0;  // then it walks on
       for (uint64_t tile = w.t0; tile < w.t1; tile += w.ts) {
         if (*(volatile int *)&abort_flag) break;
         cur = find_tile(plan, cur, tile);
@@ -524,9 +529,9 @@ __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
         uint16_t *const g = const_cast<uint16_t *>(E.g) + start;
         constexpr uint32_t kRegion = L::kES * (uint32_t)L::kTile + kPad;
         StageDesc sd{p, m, v, L::kDigests == 4 ? E.w + start : nullptr, g, cnt, E.key_base + (uint32_t)start};
-        if (MIS && E.mis) {
-          const auto off = [](const void *x) { return (uint32_t)((uintptr_t)x & 15); };
-          const auto blocks = [&](const void *x, uint32_t bytes) { return (off(x) + bytes + 15) & ~15u; };
+        const auto off = [](const void *x) { return (uint32_t)((uintptr_t)x & 15); };
+        const auto blocks = [&](const void *x, uint32_t bytes) { return (off(x) + bytes + 15) & ~15u; };
+        if (MIS && E.mis == kMisAll) {
           sd.cnt |= kMisTile | off(p) << 16 | off(m) << 20 | off(v) << 24 | off(g) << 28;
           desc[stage] = sd;
           mbar_arrive_expect_tx(&full[stage], blocks(p, cnt * L::kES) + blocks(m, cnt * L::kES) +
@@ -536,12 +541,15 @@ __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
           copy_blocks(st + 2 * kRegion, v, cnt * L::kES, &full[stage], policy);
           copy_blocks(st + 3 * kRegion, reinterpret_cast<const uint8_t *>(g), cnt * 2, &full[stage], policy);
         } else {
+          const bool half = MIS && E.mis == kMisGrad;
+          if (half) sd.cnt |= kHalfTile | off(g) << 28;
           desc[stage] = sd;
-          mbar_arrive_expect_tx(&full[stage], cnt * (3 * L::kES + 2));
+          mbar_arrive_expect_tx(&full[stage], cnt * 3 * L::kES + (half ? blocks(g, cnt * 2) : cnt * 2));
           bulk_g2s(st, p, cnt * L::kES, &full[stage], policy);
           bulk_g2s(st + kRegion, m, cnt * L::kES, &full[stage], policy);
           bulk_g2s(st + 2 * kRegion, v, cnt * L::kES, &full[stage], policy);
-          bulk_g2s(st + 3 * kRegion, g, cnt * 2, &full[stage], policy);
+          if (half) copy_blocks(st + 3 * kRegion, reinterpret_cast<const uint8_t *>(g), cnt * 2, &full[stage], policy);
+          else bulk_g2s(st + 3 * kRegion, g, cnt * 2, &full[stage], policy);
         }
         ++issued;
         if (++stage == L::kStages) {
@@ -552,12 +560,11 @@ __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
     }
     __syncwarp();
     // With its copies issued, the producer warp does what the entries hold
-    // outside their tiles, one entry at a time: up to 8 elements before
-    // (lanes 0-7) and 24 behind (lanes 8-31).
+    // outside their tiles (at most 31 elements), one entry at a time.
     for (uint32_t e = blockIdx.x; e < plan.count; e += gridDim.x) {
       const CommitEntry &E = plan.e[e];
-      const uint64_t i = lane < 8 ? lane : E.head + E.body + (lane - 8);
-      if (i < (lane < 8 ? (uint64_t)E.head : E.n)) {
+      if (lane < (uint32_t)(E.n - E.body)) {
+        const uint64_t i = lane < E.head ? lane : lane + E.body;
         L::one(E, i, s, a);
         if (ZERO) const_cast<uint16_t *>(E.g)[i] = 0;
       }
@@ -591,7 +598,7 @@ __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
       const StageDesc sd = desc[stage];
       const uint8_t *st = smem + (size_t)stage * kStage;
       if (MIS && (sd.cnt & kMisTile)) {
-        const uint32_t cnt = sd.cnt & (kMisTile - 1);
+        const uint32_t cnt = sd.cnt & kCntMask;
         const typename L::Mis x(st, sd.cnt);
         uint32_t e = ct;
 #pragma unroll L::kMisUnroll
@@ -602,11 +609,13 @@ __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
       } else {
         typename L::Regs r[L::kGroups];
         bool ok[L::kGroups];
+        const bool half = MIS && (sd.cnt & kHalfTile);
+        const uint32_t cnt = MIS ? sd.cnt & kCntMask : sd.cnt;
 #pragma unroll
         for (int k = 0; k < L::kGroups; ++k) {
           const uint32_t e = (uint32_t)(k * L::kConsumers + ct) * 4;
-          ok[k] = e < sd.cnt;
-          if (ok[k]) L::template load<kPad>(st, e, r[k]);
+          ok[k] = e < cnt;
+          if (ok[k]) L::template load<kPad>(st, e, half, sd.cnt >> 28, r[k]);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[stage]);
@@ -614,7 +623,7 @@ __global__ void __launch_bounds__(L::kBoundThreads, kCommitBlocksPerSm)
         const uint32_t ob = 4u * (uint32_t)ct;
         const Dst d{sd.p + ob * L::kES, sd.m + ob * L::kES, sd.v + ob * L::kES,
                     L::kDigests == 4 ? sd.w + ob : nullptr, sd.g + ob};
-        store_groups<L, ZERO, 0>(d, sd.G + ob, r, ok, s, a);
+        store_groups<L, ZERO, MIS, 0>(d, sd.G + ob, r, ok, half, s, a);
       }
       if (++stage == L::kStages) {
         stage = 0;

@@ -462,13 +462,16 @@ apc_status commit_common(int layout, const std::vector<TableRow> &rows, const ap
     e.w = t.w;
     e.n = t.n;
     e.key_base = (uint32_t)t.goff;
-    // aligned: whole 16-byte vectors from there on; misaligned: 8 elements left
-    // out on either side, all of them where that leaves no vector
-    const uint64_t head = std::min<uint64_t>(aligned ? h0 : 8, t.n);
+    // aligned: whole 16-byte vectors from there on.  Otherwise 8 elements are
+    // left out on either side, and the body starts where p, m and v sit on a
+    // 16-byte boundary if they do so together.
+    const uint64_t hp = ((16 - p % 16) % 16) / es;
+    const bool state = p % 16 == m % 16 && p % 16 == v % 16;
+    const uint64_t head = std::min<uint64_t>(aligned ? h0 : state ? 8 + hp : 8, t.n);
     const uint64_t room = t.n - head - (aligned ? 0 : std::min<uint64_t>(8, t.n - head));
     e.head = (uint16_t)head;
     e.body = t.n < 32 && !aligned ? 0 : room / apc::kVec * apc::kVec;
-    e.mis = !aligned && e.body;
+    e.mis = aligned || !e.body ? apc::kMisNone : state ? apc::kMisGrad : apc::kMisAll;
     entries.push_back(e);
   }
   std::vector<Range> ranges;

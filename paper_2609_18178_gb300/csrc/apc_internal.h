@@ -95,12 +95,15 @@ constexpr uint64_t commit_tile(int layout) { return layout == kLayoutBF16 ? kCom
 //   p, m, v: fp32 or bf16 state (by the launch's layout); w: the bf16 copy
 //         (fp32 layout only).
 //   head, body: elements [head, head + body) run in tiles of the plan's `tile`
-//         elements, the up to 8 before and 24 behind one by one.
-//   mis:  the buffers are not mutually 16-byte aligned.  Then the blocks of 16
-//         bytes that hold the body reach at most 15 bytes over it, which
-//         stays inside the buffers (8 elements are left out on either side).
+//         elements, the others (at most 31) one by one.
+//   mis:  which buffers are not 16-byte aligned at the body's start: none, g
+//         and w (kMisGrad), or any (kMisAll).  Such a buffer is read in the
+//         16-byte blocks that hold it, which reach at most 15 bytes over the
+//         body on either side; 8 elements are left out there, so the blocks
+//         stay inside the buffer.
 //   tile_begin: the entry's first tile in the launch's tile space.
 //   key_base: global_offset mod 2^32 (the digest key of element 0).
+enum CommitMis : uint16_t { kMisNone, kMisGrad, kMisAll };
 struct CommitEntry {
   void *p, *m, *v;
   const uint16_t *g;

@@ -150,7 +150,8 @@ def state_words(n, goff, step, layout):
 
 
 # Elements per tile of the commit kernel and the sizes around its edges; a
-# misaligned entry runs 8 elements on either side and entries under 32 apart.
+# misaligned entry runs 8 to 15 elements on either side, and one under 32
+# elements all of them, apart.
 TILE = {"f32": 4864, "bf16": 10368}
 
 
@@ -158,8 +159,8 @@ TILE = {"f32": 4864, "bf16": 10368}
 @pytest.mark.parametrize("layout", ["f32", "bf16"])
 def test_commit_misaligned_entries(layout, zero):
     """Entries whose buffers sit at different offsets from a 16-byte boundary,
-    of every size near the path's edges, mixed with aligned ones; nothing
-    outside a buffer changes."""
+    all of them or the gradient and copy against the state, of every size near
+    the path's edges, mixed with aligned ones; nothing outside a buffer changes."""
     rng = np.random.default_rng(21)
     t = TILE[layout]
     sizes = list(range(1, 12)) + [15, 16, 23, 24, 25, 31, 32, 33, 39, 40, 41, 1000, t - 1, t, t + 1, t + 15, t + 16, t + 17,
@@ -173,6 +174,9 @@ def test_commit_misaligned_entries(layout, zero):
         for k in "pmvgw":
             shifts[(i, k)] = same if i % 5 == 4 else int(rng.integers(0, 16))
     committed(tensors, offs, 4, layout, zero, shifts)
+    for (i, k) in shifts:
+        shifts[(i, k)] = shifts[(i, "p")] if k in "mv" else shifts[(i, k)]
+    committed(tensors, offs, 4, layout, zero, shifts)
 
 
 @pytest.mark.parametrize("layout", ["f32", "bf16"])
@@ -183,8 +187,9 @@ def test_commit_every_relative_offset(layout):
     t = state_words(n, 12345, 9, layout)
     for gs in range(8):
         for ps in range(0, 4 if layout == "f32" else 8):
-            committed([t], [12345], 9, layout, False,
-                      {(0, "p"): ps, (0, "m"): (ps + gs) % 8, (0, "v"): 3, (0, "g"): gs, (0, "w"): (gs + 1) % 8})
+            for m, v in (((ps + gs) % 8, 3), (ps, ps)):
+                committed([t], [12345], 9, layout, False,
+                          {(0, "p"): ps, (0, "m"): m, (0, "v"): v, (0, "g"): gs, (0, "w"): (gs + 1) % 8})
 
 
 @pytest.mark.parametrize("layout", ["f32", "bf16"])
