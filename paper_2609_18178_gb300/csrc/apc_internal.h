@@ -75,12 +75,6 @@ constexpr int kCommitBlocksPerSm = APC_COMMIT_BLOCKS_PER_SM;
 #ifndef APC_SMEM_CARVEOUT
 #define APC_SMEM_CARVEOUT -1
 #endif
-// Tile order of the commit kernel: 1 = CTA b takes one contiguous run of
-// tiles (the runs differ by at most one tile), 0.3-0.7% faster than 0 = CTA b
-// takes tiles b, b + grid, ... (the grid sweeping the table together).
-#ifndef APC_COMMIT_CONTIGUOUS
-#define APC_COMMIT_CONTIGUOUS 1
-#endif
 // A stage holds one tile of p, m, v and g: 14 bytes per element for fp32
 // state (66.5 KB, 200 KB per CTA at the defaults), 8 for bf16 state (81 KB,
 // 162 KB per CTA).
