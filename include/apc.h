@@ -48,12 +48,14 @@
  *   - Device pointers belong to the calling thread's current CUDA device:
  *     every buffer a kernel reads or writes, and every output, must be
  *     device memory of that device (or managed memory).  Each call checks
- *     this with one cudaPointerGetAttributes query per distinct address and
- *     returns APC_EINVAL for host memory or another device's memory.
+ *     this with one cudaPointerGetAttributes query per allocation (per
+ *     distinct address where the driver gives no single range) and returns
+ *     APC_EINVAL for host memory or another device's memory.
  *     The caller owns all memory and the library allocates nothing.  Between
  *     calls it keeps only each device's SM count and kernel residency
- *     (queried once), the kernels' device status word (apc_device_status)
- *     and the number of SMs to leave free (apc_set_reserved_sms).
+ *     (queried once), the kernels' device status word (apc_device_status),
+ *     the number of SMs to leave free (apc_set_reserved_sms) and the locks
+ *     that keep two threads' chains of launches on one stream apart.
  *   - Work is enqueued on `stream` (NULL = the legacy default stream); the
  *     call never synchronizes.  Results, including the digests, are valid
  *     once the stream reaches that point.
@@ -102,8 +104,9 @@ typedef struct apc_adamw_hparams {
  *   w        bf16 bits, device, n elements, written (p' rounded to bf16)
  *   global_offset  index of element 0 in the flat model (the digest key)
  * p, m, v need 4-byte and g, w 2-byte alignment; the kernel runs 16-byte
- * vectors wherever the five buffers are mutually aligned and scalar code
- * elsewhere.  n == 0 entries are skipped and their pointers may be NULL.
+ * vectors on p, m and v where those are mutually aligned, and on g and w where
+ * these are so too, and element accesses elsewhere.  n == 0 entries are skipped
+ * and their pointers may be NULL.
  * The written ranges of all entries (p, m, v, w) must not overlap each other
  * or any gradient range. */
 typedef struct apc_tensor {

@@ -1,10 +1,11 @@
 // Device arithmetic of the committed step: the AdamW element update in its
 // fixed binary32 order and the splitmix64 digest term.
 //
-// Every floating-point operation is an explicit round-to-nearest intrinsic
-// (__fmul_rn, __fadd_rn, __fsub_rn, __fsqrt_rn, __fdiv_rn), which the
-// compiler never fuses into FMA; the library is also built with -fmad=false
-// and without flush-to-zero.  The update is decoupled-weight-decay AdamW
+// Every result is that of separate round-to-nearest operations (__fmul_rn,
+// __fadd_rn, __fsub_rn, __fsqrt_rn, __fdiv_rn), which the compiler never fuses
+// into FMA; the library is also built with -fmad=false and without
+// flush-to-zero.  adamw_group forms the same square roots and quotients from
+// approximations with exact remainders.  The update is decoupled-weight-decay AdamW
 // (the optimizer whose committed W, M, V the paper preserves, arxiv
 // 2609.18178 Section III-A, Eq. 2) and the digest realises its bitwise rank
 // state checks (Sections IV-F, IV-G).
