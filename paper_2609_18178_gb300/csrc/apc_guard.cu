@@ -15,11 +15,12 @@
 // walk it interleaved, each on its own.  A lane issues all its kCountGroups
 // 16-byte loads of a tile before it counts, group j of a warp being 512
 // consecutive bytes.  What a buffer holds beyond its full tiles goes to one
-// warp, before the walks.
+// warp, before the walks: the CTA's last warps first, as the walk deals them one
+// tile fewer (152 M in 146 tensors 50.9 us; 51.4 from the first warp on).
 //
 // Tiles of a whole CTA (64 KB, dealt out round robin) made its 1,024 threads
 // wait for one tile at a time.  Against that, calls over bf16 gradients take:
-// 152 M in 146 tensors 53 us (62), 2 M in 100 tensors 9.8 (26), 7.25 G in 291
+// 152 M in 146 tensors 51 us (62), 2 M in 100 tensors 9.8 (26), 7.25 G in 291
 // tensors 1,972 (2,158), which is 7.35 TB/s.
 #include <cuda_runtime.h>
 
@@ -55,7 +56,7 @@ __global__ void __launch_bounds__(kCountThreads, 1) count_kernel(const __grid_co
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // what the entries hold beyond their full tiles: the body's last groups, and
   // the scalar head (lanes 0-6) and tail (lanes 8-14)
-  for (uint32_t e = blockIdx.x + gridDim.x * warp; e < plan.count; e += gridDim.x * kWarps) {
+  for (uint32_t e = blockIdx.x + gridDim.x * (kWarps - 1 - warp); e < plan.count; e += gridDim.x * kWarps) {
     const DigestEntry &E = plan.e[e];
     const bool f32 = E.dtype == 0;
     const uint32_t es = f32 ? 4 : 2;
