@@ -14,6 +14,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "apc_internal.h"
 
 namespace apc {
@@ -297,7 +299,11 @@ __device__ __forceinline__ Key16 key16(uint32_t gidx, uint32_t one, uint32_t top
 // Term of half HALF (0 low, 1 high) of the packed words `pair`.  The half is
 // taken and the increment added by one two-way dot product (dp2a with a unit
 // vector), in place of a mask or shift and an add (4,234 to 4,065 us over
-// 1.81 G elements of bf16 state).
+// 1.81 G elements of bf16 state).  The second multiply is the compiler's
+// for the high halves and three multiply-adds for the low ones: with both
+// integer pipes 77% busy that mix lets them interleave best (3,650 us; 3,669
+// with multiply-adds for both, 3,681 with the compiler's for both, 3,741 with
+// the two exchanged).
 template <uint32_t OFF, int HALF>
 __device__ __forceinline__ uint64_t digest_term_u16(const Key16 &k, uint32_t pair) {
   static_assert(OFF % 4 == 0, "a Key16 serves offsets of its own residue mod 4");
@@ -312,7 +318,7 @@ __device__ __forceinline__ uint64_t digest_term_u16(const Key16 &k, uint32_t pai
       "mov.b64 %0, {rl, rh};\n\t}"
       : "=l"(z)
       : "r"(l1), "n"(0x1CE4E5B9u), "n"(0xBF58476Du), "r"(k.t + OFF * 0x1CE4E5B9u));
-  z = MulWide::template mul<0x133111EBu, 0x94D049BBu>(z ^ (z >> 27));
+  z = std::conditional<HALF == 1, MulCompiler, MulWide>::type::template mul<0x133111EBu, 0x94D049BBu>(z ^ (z >> 27));
   return z ^ (z >> 31);
 }
 
