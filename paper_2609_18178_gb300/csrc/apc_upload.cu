@@ -9,8 +9,12 @@
 // in the digest kernel (one contiguous run of the launch's tiles per CTA, its
 // warps interleaved).  Each lane issues all of its kUploadGroups loads of a
 // tile before any store, which keeps enough bytes in flight to cover the
-// link's latency.  What a segment holds beyond its full tiles is done by one
-// warp before the walks.
+// link's latency.  What a segment holds beyond its full tiles is done before the
+// walks, by the CTAs' last warps first, which a short launch leaves without a
+// tile, the bytes at a segment's ends and its last words by two different
+// warps: every part then waits for the link once.  In 7 segments of a packed
+// bucket 600 KB take 8.1 us and 2 MB 14.2 (12.4 and 19.7 with one of the first
+// warps per segment, 12.2 and 25 when every byte was copied alone).
 //
 // A segment whose source and destination are not mutually 16-byte aligned (an
 // odd-sized tensor in a packed host bucket) is read in the 16-byte blocks of
@@ -18,7 +22,7 @@
 // and the next lane's, which comes by shuffle.  The blocks reach up to 15 bytes
 // over the words, so 15 to 31 bytes at the start and at least 16 at the end of
 // such a segment are copied byte by byte.  40 MB in 146 segments of a packed
-// bucket take 200 us (428 when every byte of such a segment was copied alone;
+// bucket take 198 us (428 when every byte of such a segment was copied alone;
 // 190 at the link's 211 GB/s), 1 GB in 20 segments on 16 CTAs 4.8 ms (97.7).
 #include <cuda_runtime.h>
 
@@ -58,25 +62,40 @@ __device__ __forceinline__ uint4 next_lane(const uint4 &x, uint32_t lane) {
 // end-to-end step of 14.5 GB of gradients took 79.6 ms instead of 69.2.
 __global__ void __launch_bounds__(kUploadThreads, 2) upload_kernel(const __grid_constant__ UploadPlan<kUploadMax> plan) {
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // what the segments hold beyond their full tiles
-  for (uint32_t e = blockIdx.x + gridDim.x * warp; e < plan.count; e += gridDim.x * kWarps) {
-    const UploadEntry &E = plan.e[e];
-    for (uint64_t i = lane; i < E.head; i += 32) E.dst[i] = E.src[i];
-    for (uint64_t i = E.head + E.body + lane; i < E.bytes; i += 32) E.dst[i] = E.src[i];
+  // what the segments hold beyond their full tiles, the bytes at the ends and the
+  // last words each by a warp of its own
+  for (uint32_t i = blockIdx.x + gridDim.x * (kWarps - 1 - warp); i < 2 * plan.count; i += gridDim.x * kWarps) {
+    const UploadEntry &E = plan.e[i >> 1];
+    if (i & 1) {
+      const uint64_t end = E.head + E.body;
+      const uint32_t rest = (uint32_t)(E.bytes - end);  // under 32; the head is under 64
+      uint8_t b0 = 0, b1 = 0, b2 = 0;
+      if (lane < E.head) b0 = E.src[lane];
+      if (lane + 32 < E.head) b1 = E.src[lane + 32];
+      if (lane < rest) b2 = E.src[end + lane];
+      if (lane < E.head) E.dst[lane] = b0;
+      if (lane + 32 < E.head) E.dst[lane + 32] = b1;
+      if (lane < rest) E.dst[end + lane] = b2;
+      continue;
+    }
     const uint64_t at = E.head + E.body / kUploadTile * kUploadTile;
     const uint4 *src = reinterpret_cast<const uint4 *>(E.src + at - E.shift);
     uint4 *dst = reinterpret_cast<uint4 *>(E.dst + at);
     const uint32_t words = (uint32_t)(E.body % kUploadTile) / 16;
     // all loads first here too: one latency of the link, not one per word
-    uint4 x[kUploadGroups];
-    if (E.shift == 0) {
+    const uint32_t shift = E.shift, blocks = words + (shift != 0);  // at most 256
+    uint4 x[kUploadGroups] = {};
 #pragma unroll
-      for (int j = 0; j < kUploadGroups; ++j)
-        if (j * 32 + lane < words) x[j] = __ldcs(src + j * 32 + lane);
-    } else {
+    for (int j = 0; j < kUploadGroups; ++j)
+      if (j * 32 + lane < blocks) x[j] = __ldcs(src + j * 32 + lane);
+    if (shift != 0) {
+      uint4 n = next_lane(x[0], lane);
 #pragma unroll
-      for (int j = 0; j < kUploadGroups; ++j)
-        if (j * 32 + lane < words) x[j] = cut(__ldcs(src + j * 32 + lane), __ldcs(src + j * 32 + lane + 1), E.shift);
+      for (int j = 0; j < kUploadGroups; ++j) {
+        const uint4 after = j + 1 < kUploadGroups ? next_lane(x[j + 1], lane) : n;
+        x[j] = cut(x[j], lane < 31 ? n : after, shift);
+        n = after;
+      }
     }
 #pragma unroll
     for (int j = 0; j < kUploadGroups; ++j)
@@ -85,13 +104,13 @@ __global__ void __launch_bounds__(kUploadThreads, 2) upload_kernel(const __grid_
   // this CTA's run of tiles, walked by its warps
   const uint64_t per = plan.total_tiles / gridDim.x, rem = plan.total_tiles % gridDim.x;
   const uint64_t t_begin = blockIdx.x * per + (blockIdx.x < rem ? blockIdx.x : rem);
-  const uint64_t len = per + (blockIdx.x < rem ? 1 : 0);
+  const uint32_t len = (uint32_t)(per + (blockIdx.x < rem ? 1 : 0));  // 2^32 tiles are 16 TB
   uint32_t cur = 0;
-  for (uint64_t r = warp; r < len;) {
+  for (uint32_t r = warp; r < len;) {
     cur = entry_of(plan, cur, t_begin + r);
     const UploadEntry &E = plan.e[cur];
     const uint64_t left = (cur + 1 < plan.count ? plan.e[cur + 1].tile_begin : plan.total_tiles) - t_begin;
-    const uint64_t stop = left < len ? left : len;
+    const uint32_t stop = left < len ? (uint32_t)left : len;
     const uint64_t at = E.head + (t_begin + r - E.tile_begin) * kUploadTile;
     const uint32_t shift = E.shift;
     const uint4 *src = reinterpret_cast<const uint4 *>(E.src + at - shift) + lane;
