@@ -185,7 +185,10 @@ apc_status with_plan(size_t count, F f) {
 
 // The launches of a long table go onto their stream as one chain (launch_plan):
 // a chain of another thread on the same stream must not mix with them.  (A
-// single launch may come in between: it starts nothing early.)
+// single launch may come in between: it starts nothing early.)  Only where the
+// grid may take the whole GPU: the next launch's CTAs would otherwise start on
+// the SMs that the caller keeps free (apc_set_reserved_sms, APC_GRID_LIMIT) and
+// hold them until the launch before has ended.
 std::mutex &chain_lock(const void *stream) {
   static std::mutex locks[64];
   const uintptr_t s = (uintptr_t)stream;
@@ -197,16 +200,23 @@ std::atomic<int> g_reserved_sms{0};
 
 // The persistent grid: one CTA per resident slot on the SMs not reserved
 // (at least one SM's worth), capped by APC_GRID_LIMIT (read at every call)
-// when that is a positive integer.
-unsigned grid_for(uint64_t tiles, int sms, int per_sm) {
+// when that is a positive integer.  `whole`: neither leaves a slot free.  Read
+// once a call, so that all its launches agree.
+struct Grid {
+  unsigned cap;
+  bool whole;
+};
+
+Grid grid_for(int sms, int per_sm) {
   const int avail = std::max(1, sms - g_reserved_sms.load(std::memory_order_relaxed));
-  uint64_t cap = (uint64_t)avail * (uint64_t)std::max(per_sm, 1);
+  const uint64_t slots = (uint64_t)std::max(per_sm, 1);
+  uint64_t cap = (uint64_t)avail * slots;
   if (const char *lim = std::getenv("APC_GRID_LIMIT")) {
     char *end = nullptr;
     const unsigned long long v = std::strtoull(lim, &end, 10);
     if (end != lim && *end == 0 && v > 0) cap = std::min<uint64_t>(cap, v);
   }
-  return (unsigned)std::max<uint64_t>(1, std::min(tiles, cap));
+  return {(unsigned)cap, cap == (uint64_t)sms * slots};
 }
 
 // The address range of the allocation that holds `p`, if it is an ordinary
@@ -339,17 +349,18 @@ void commit_scalars(const float h[8], apc::CommitPlan<MAXE> *plan) {
 // Entries arrive without tile_begin; each batch places their tiles.
 template <int MAXE, typename Launch>
 apc_status run_commit_batches(const std::vector<apc::CommitEntry> &entries, const float h[8], int layout,
-                              bool zero_grad, unsigned grid_cap, void *stream, unsigned long long *out,
+                              bool zero_grad, Grid grid_max, void *stream, unsigned long long *out,
                               Launch launch) {
   std::unique_ptr<apc::CommitPlan<MAXE>> plan(new apc::CommitPlan<MAXE>);  // not cleared: the kernel reads what is filled
   commit_scalars(h, plan.get());
   plan->one = 1;
-  std::unique_lock<std::mutex> chain;
-  if (entries.size() > (size_t)MAXE) chain = std::unique_lock<std::mutex>(chain_lock(stream));
+  const bool chain = grid_max.whole && entries.size() > (size_t)MAXE;
+  std::unique_lock<std::mutex> lock;
+  if (chain) lock = std::unique_lock<std::mutex>(chain_lock(stream));
   size_t i = 0;
   while (i < entries.size()) {
     const size_t k = std::min(entries.size() - i, (size_t)MAXE);
-    const uint32_t tile = commit_launch_tile(&entries[i], k, apc::commit_tile(layout), grid_cap);
+    const uint32_t tile = commit_launch_tile(&entries[i], k, apc::commit_tile(layout), grid_max.cap);
     uint64_t tiles = 0;
     for (size_t j = 0; j < k; ++j) {
       apc::CommitEntry e = entries[i + j];
@@ -360,10 +371,10 @@ apc_status run_commit_batches(const std::vector<apc::CommitEntry> &entries, cons
     plan->tile = tile;
     plan->count = (uint32_t)k;
     plan->total_tiles = tiles;
-    plan->more = i + k < entries.size();
-    plan->chained = i > 0;
+    plan->more = chain && i + k < entries.size();
+    plan->chained = chain && i > 0;
     const uint64_t want = std::max<uint64_t>(tiles, k);
-    const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(want, grid_cap));
+    const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(want, grid_max.cap));
     int e = launch(*plan, layout, zero_grad, grid, stream, out);
     if (e) return cuda_fail(e, "commit kernel launch");
     i += k;
@@ -374,12 +385,13 @@ apc_status run_commit_batches(const std::vector<apc::CommitEntry> &entries, cons
 // Entries arrive with the element count of their vector body in tile_begin;
 // tiles_of(body, element size) is the kernel's count of whole tiles in it.
 template <int MAXE, typename Tiles, typename Launch>
-apc_status run_digest_batches(const std::vector<apc::DigestEntry> &entries, unsigned grid_cap, const void *stream,
+apc_status run_digest_batches(const std::vector<apc::DigestEntry> &entries, Grid grid_max, const void *stream,
                               Tiles tiles_of, Launch launch, const char *what) {
   std::unique_ptr<apc::DigestPlan<MAXE>> plan(new apc::DigestPlan<MAXE>);
   plan->one = 1;
-  std::unique_lock<std::mutex> chain;
-  if (entries.size() > (size_t)MAXE) chain = std::unique_lock<std::mutex>(chain_lock(stream));
+  const bool chain = grid_max.whole && entries.size() > (size_t)MAXE;
+  std::unique_lock<std::mutex> lock;
+  if (chain) lock = std::unique_lock<std::mutex>(chain_lock(stream));
   size_t i = 0;
   while (i < entries.size()) {
     const size_t k = std::min(entries.size() - i, (size_t)MAXE);
@@ -395,9 +407,9 @@ apc_status run_digest_batches(const std::vector<apc::DigestEntry> &entries, unsi
     plan->count = (uint32_t)k;
     plan->total_tiles = tiles;
     plan->tiles32 = tiles32;
-    plan->more = i + k < entries.size();
-    plan->chained = i > 0;
-    const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(std::max<uint64_t>(tiles, k), grid_cap));
+    plan->more = chain && i + k < entries.size();
+    plan->chained = chain && i > 0;
+    const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(std::max<uint64_t>(tiles, k), grid_max.cap));
     int e = launch(*plan, grid);
     if (e) return cuda_fail(e, what);
     i += k;
@@ -500,9 +512,9 @@ apc_status commit_common(int layout, const std::vector<TableRow> &rows, const ap
   int e = (int)cudaMemsetAsync(out, 0, (size_t)nslots * sizeof(uint64_t), (cudaStream_t)stream);
   if (e) return cuda_fail(e, "cudaMemsetAsync(out_digests)");
   if (entries.empty()) return APC_OK;
-  const unsigned cap = grid_for(UINT64_MAX, d.sms, d.commit);
+  const Grid grid_max = grid_for(d.sms, d.commit);
   return with_plan<apc::kCommitSmall, apc::kCommitMid, apc::kCommitLarge>(entries.size(), [&](auto size) {
-    return run_commit_batches<size.value>(entries, h, layout, zero_grad, cap, stream, out,
+    return run_commit_batches<size.value>(entries, h, layout, zero_grad, grid_max, stream, out,
                                           apc::launch_commit<size.value>);
   });
 }
@@ -609,17 +621,17 @@ APC_EXPORT apc_status apc_digest(const apc_buffer *bufs, int32_t num_bufs, int32
   int e = (int)cudaMemsetAsync(out, 0, (size_t)num_slots * sizeof(uint64_t), (cudaStream_t)stream);
   if (e) return cuda_fail(e, "cudaMemsetAsync(out_digests)");
   if (entries.empty()) return APC_OK;
-  const unsigned cap = grid_for(UINT64_MAX, d.sms, d.digest);
+  const Grid grid_max = grid_for(d.sms, d.digest);
   // long tiles where every warp of the grid gets several of them in a launch
   uint64_t body = 0;
   for (const apc::DigestEntry &en : entries) body += en.tile_begin;
-  const uint64_t warps = (uint64_t)cap * (apc::kThreads / 32);
+  const uint64_t warps = (uint64_t)grid_max.cap * (apc::kThreads / 32);
   const uint64_t launches = ceil_div(entries.size(), apc::kDigestLarge);
   const int u = body / apc::digest_tile(apc::kDigestLong) >= apc::kDigestLongTiles * warps * launches ? apc::kDigestLong
                                                                                                        : apc::kDigestShort;
   return with_plan<apc::kDigestSmall, apc::kDigestMid, apc::kDigestLarge>(entries.size(), [&](auto size) {
     return run_digest_batches<size.value>(
-        entries, cap, stream, [u](uint64_t n, uint64_t) { return n / apc::digest_tile(u); },
+        entries, grid_max, stream, [u](uint64_t n, uint64_t) { return n / apc::digest_tile(u); },
         [&](const auto &plan, unsigned grid) { return apc::launch_digest(plan, u, grid, stream, out); },
         "digest kernel launch");
   });
@@ -637,10 +649,10 @@ APC_EXPORT apc_status apc_count_nonzero(const apc_buffer *bufs, int32_t num_bufs
   int e = (int)cudaMemsetAsync(out, 0, (size_t)num_slots * sizeof(uint64_t), (cudaStream_t)stream);
   if (e) return cuda_fail(e, "cudaMemsetAsync(out_counts)");
   if (entries.empty()) return APC_OK;
-  const unsigned cap = grid_for(UINT64_MAX, d.sms, d.count);
+  const Grid grid_max = grid_for(d.sms, d.count);
   return with_plan<apc::kDigestSmall, apc::kDigestMid, apc::kDigestLarge>(entries.size(), [&](auto size) {
     return run_digest_batches<size.value>(
-        entries, cap, stream, [](uint64_t n, uint64_t es) { return n * es / apc::kCountTileBytes; },
+        entries, grid_max, stream, [](uint64_t n, uint64_t es) { return n * es / apc::kCountTileBytes; },
         [&](const auto &plan, unsigned grid) { return apc::launch_count(plan, grid, stream, out); },
         "count kernel launch");
   });

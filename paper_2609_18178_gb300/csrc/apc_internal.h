@@ -131,8 +131,8 @@ struct CommitPlan {
   uint32_t count;
   uint32_t one;          // 1: the FMA-pipe carry-add multiplier of the digest
   uint32_t tile;         // elements per tile of this launch (a multiple of 64, at most commit_tile)
-  uint16_t more;         // another launch of the same call follows
-  uint16_t chained;      // this one follows another of the same call
+  uint16_t more;         // another launch of the same call follows, chained to this one
+  uint16_t chained;      // this one is chained to another of the same call before it
   CommitEntry e[MAXE];
 };
 
@@ -210,8 +210,8 @@ struct DigestPlan {
   uint64_t tiles32;      // tiles of the fp32 entries, which come first (digest kernel)
   uint32_t count;
   uint32_t one;          // 1: the FMA-pipe carry-add multiplier of the digest
-  uint16_t more;         // another launch of the same call follows
-  uint16_t chained;      // this one follows another of the same call
+  uint16_t more;         // another launch of the same call follows, chained to this one
+  uint16_t chained;      // this one is chained to another of the same call before it
   uint32_t pad_;
   DigestEntry e[MAXE];
 };

@@ -169,3 +169,46 @@ def test_upload_commit_digest_captured_in_one_graph():
         assert apc.digests_to_host(out_v) == dref
         for d, r in zip(devs, ref):
             assert np.array_equal(d["g"].cpu().numpy().view(np.uint16), r["g"])
+
+
+@pytest.mark.parametrize("what", ["commit", "verify"])
+def test_upload_on_reserved_sms_beside_a_long_table(what):
+    """A call of two launches, the first of them long, leaves the reserved SMs
+    free all the while: an upload enqueued after it on another stream is done
+    before half of the call's time has passed."""
+    n, k = 1 << 20, 440 if what == "commit" else 250
+    f32 = lambda: torch.zeros((k + 40) * n, dtype=torch.float32, device="cuda")
+    f16 = lambda: torch.zeros((k + 40) * n, dtype=torch.int16, device="cuda")
+    b = dict(p=f32(), m=f32(), v=f32(), g=f16(), w=f16())
+    e = []
+    for i in range(k + 40):
+        size = n if i < k else 256          # the second launch: 40 short entries, work for 40 CTAs
+        e.append(apc.TensorEntry(*(b[f][i * n:i * n + size] for f in "pmvgw"), i * n))
+    if what == "commit":
+        table = apc.prepare_table(e)
+        call = lambda s: apc.commit_step(table, 1, stream=s, out=out)
+    else:
+        bufs = [apc.BufferEntry(getattr(t, f), 0, t.global_offset, apc.F32) for t in e for f in "pmv"]
+        bufs += [apc.BufferEntry(t.g, 0, t.global_offset, apc.BF16) for t in e]
+        table = apc.prepare_buffers(bufs)
+        call = lambda s: apc.digest(table, 4, stream=s, out=out)
+    out = torch.zeros(4, dtype=torch.int64, device="cuda")
+    h = pinned_bytes(1 << 20, 9)
+    seg = apc.prepare_segments([apc.Segment(torch.empty(1 << 20, dtype=torch.uint8, device="cuda"), h)])
+    s, side = torch.cuda.Stream(), torch.cuda.Stream()
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(3)]
+    try:
+        apc.set_reserved_sms(8)
+        for timed in (False, True):          # the first time loads the kernels
+            torch.cuda.synchronize()
+            ev[0].record(s)
+            call(s)
+            ev[1].record(s)
+            apc.upload(seg, 16, stream=side)
+            ev[2].record(side)
+            torch.cuda.synchronize()
+        whole, uploaded = ev[0].elapsed_time(ev[1]), ev[0].elapsed_time(ev[2])
+        print("%s of %d entries: call %.3f ms, upload done at %.3f ms" % (what, len(e), whole, uploaded))
+        assert uploaded < 0.5 * whole
+    finally:
+        apc.set_reserved_sms(0)

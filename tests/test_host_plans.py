@@ -1,0 +1,82 @@
+"""The launches that the library's host side makes of a call, on the CPU:
+csrc/apc_host.cpp is compiled as it is against a stand-in for the CUDA
+runtime and the kernels (host_stub.cpp) that records what it is asked."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import pytest
+
+import oracle
+import paper_2609_18178_gb300 as apc
+from paper_2609_18178_gb300 import _build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+BASE = 1 << 40   # fake device addresses, one GB apart per kind of buffer
+SMS = 152
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    nvcc = shutil.which(os.environ.get("NVCC", "nvcc")) or "/usr/local/cuda/bin/nvcc"
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
+    so = str(tmp_path_factory.mktemp("host") / "libhost.so")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-fvisibility=hidden", "-Wl,-Bsymbolic", "-I", cuda,
+                    "-I", _build.CSRC, os.path.join(_build.CSRC, "apc_host.cpp"), os.path.join(HERE, "host_stub.cpp"),
+                    "-o", so], check=True)
+    out = ctypes.CDLL(so)
+    out.apc_last_error.restype = ctypes.c_char_p
+    for f in (out.stub_runtime_queries, out.stub_range_queries, out.stub_launches):
+        f.restype = ctypes.c_long
+    out.stub_reset.argtypes = [ctypes.c_uint64, ctypes.c_int]
+    yield out
+    out.apc_set_reserved_sms(0)
+
+
+def call(lib, what, count, n=300):
+    """One call over `count` tensors or buffers of n elements each; its status."""
+    out = ctypes.c_void_p(BASE + (7 << 30))
+    if what == "commit":
+        h = oracle.DEFAULT_HP
+        hp = apc._HParams(h["lr"], h["beta1"], h["beta2"], h["eps"], h["weight_decay"])
+        arr = (apc._Tensor * count)()
+        for k in range(count):
+            at = [BASE + (i << 30) + (4 if i < 3 else 2) * k * (n + 4) for i in range(5)]
+            arr[k] = apc._Tensor(*at, n, k * n)
+        return lib.apc_commit_step(arr, count, ctypes.byref(hp), ctypes.c_int64(3), None, out)
+    arr = (apc._Buffer * count)()
+    for k in range(count):
+        arr[k] = apc._Buffer(BASE + 4 * k * (n + 4), n, k * n, apc.F32, 0)
+    return (lib.apc_digest if what == "digest" else lib.apc_count_nonzero)(arr, count, 1, None, out)
+
+
+def launches(lib):
+    buf = (ctypes.c_int64 * 64)()
+    k = lib.stub_launches(buf, 16)
+    return [dict(zip(("count", "grid", "more", "chained"), buf[4 * i:4 * i + 4])) for i in range(k)]
+
+
+PER_SM = dict(commit=1, digest=1, count=2)   # resident CTAs, as the stand-in answers
+
+
+@pytest.mark.parametrize("what,count", [("commit", 1100), ("digest", 2300), ("count", 2300)])
+@pytest.mark.parametrize("reserved,limit", [(0, None), (8, None), (0, 20), (0, 10_000), (151, 1)])
+def test_long_tables_leave_the_sms_free_that_they_are_told_to(lib, monkeypatch, what, count, reserved, limit):
+    """A launch that lets the next one start early hands it every SM that is
+    free, also those that the grid's cap was to leave free: a call's launches
+    are chained only where their grid may take the whole GPU."""
+    monkeypatch.delenv("APC_GRID_LIMIT", raising=False)
+    if limit:
+        monkeypatch.setenv("APC_GRID_LIMIT", str(limit))
+    lib.stub_reset(0, 0)
+    assert lib.apc_set_reserved_sms(reserved) == 0
+    assert call(lib, what, count) == 0
+    got = launches(lib)
+    assert len(got) == 3 and sum(x["count"] for x in got) == count
+    whole = SMS * PER_SM[what]
+    cap = min((SMS - reserved) * PER_SM[what], limit or whole)
+    assert all(x["grid"] <= cap for x in got)
+    chained = cap == whole
+    assert [x["more"] for x in got] == [int(chained)] * 2 + [0]
+    assert [x["chained"] for x in got] == [0] + [int(chained)] * 2
