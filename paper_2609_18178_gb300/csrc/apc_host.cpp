@@ -249,16 +249,20 @@ bool allocation_of(const void *p, uintptr_t *lo, uintptr_t *hi) {
 // memory, or host memory, would otherwise be dereferenced by this device's
 // copies.  In address order, one attribute query per allocation where its
 // range is known, and one per distinct address otherwise: 1,100 tensors' 5,500
-// pointers in five arenas take 6 queries instead of 5,500 (0.14 us each).
-// Nothing is kept from one call to the next.  Returns APC_ECUDA if the runtime
-// cannot answer (for example, no device) and APC_EINVAL naming the first
-// foreign pointer (lowest address first).
+// pointers in five arenas take 6 queries instead of 5,500 (0.14 us each).  After
+// a failed range query the next 1, 2, 4, ... addresses are taken one by one
+// before a range is asked for again, so that a table in virtual memory costs at
+// most log2 of its length more than its addresses (5,500 of them in PyTorch's
+// expandable segments: 850 us a commit, 1,450 with a range query for each).  Nothing is kept from one call to the next.  Returns APC_ECUDA
+// if the runtime cannot answer (for example, no device) and APC_EINVAL naming
+// the first foreign pointer (lowest address first).
 apc_status check_device_pointers(const Ordered &ranges, size_t count, const char *out_name) {
   constexpr size_t kFew = 8;  // fewer pointers than this are queried one by one
   int dev = 0;
   int e = (int)cudaGetDevice(&dev);
   if (e) return cuda_fail(e, "cudaGetDevice");
-  uintptr_t lo = 0, hi = 0;  // the allocation last queried
+  uintptr_t lo = 0, hi = 0;     // the allocation last queried
+  size_t one_by_one = 0, next = 1;  // addresses until a range is asked for again, and after the next failure
   apc_status st = APC_OK;
   ranges.each([&](const Range &o) {
     if (o.lo >= lo && o.lo < hi) return true;
@@ -281,10 +285,17 @@ apc_status check_device_pointers(const Ordered &ranges, size_t count, const char
                 (int)a.type, a.device);
       return false;
     }
-    if (count < kFew || a.type != cudaMemoryTypeDevice || !allocation_of(p, &lo, &hi)) {
-      lo = o.lo;
-      hi = o.lo + 1;
+    if (count >= kFew && a.type == cudaMemoryTypeDevice) {
+      if (one_by_one) {
+        --one_by_one;
+      } else {
+        if (allocation_of(p, &lo, &hi)) return true;
+        one_by_one = next;
+        next *= 2;
+      }
     }
+    lo = o.lo;
+    hi = o.lo + 1;
     return true;
   });
   return st;

@@ -80,3 +80,21 @@ def test_long_tables_leave_the_sms_free_that_they_are_told_to(lib, monkeypatch, 
     chained = cap == whole
     assert [x["more"] for x in got] == [int(chained)] * 2 + [0]
     assert [x["chained"] for x in got] == [0] + [int(chained)] * 2
+
+
+@pytest.mark.parametrize("what,count,addresses,arenas", [("commit", 1100, 5501, 6), ("digest", 2300, 2301, 2), ("count", 2300, 2301, 2)])
+@pytest.mark.parametrize("virtual", ["none", "all", "some"])
+def test_pointer_queries_by_kind_of_memory(lib, what, count, addresses, arenas, virtual):
+    """One attribute query and one range query per allocation of cudaMalloc's.
+    Memory of the virtual-memory interface is asked address by address, and the
+    failed range queries beside that stay a handful, however long the table; a
+    list that begins in such memory still finds its way back."""
+    lib.stub_reset({"none": 0, "all": 1 << 63, "some": BASE + (1 << 30)}[virtual], 0)
+    assert call(lib, what, count) == 0
+    asked, ranges = lib.stub_runtime_queries(), lib.stub_range_queries()
+    if virtual == "none":
+        assert asked == ranges == arenas
+    elif virtual == "all":
+        assert asked == addresses and ranges <= 13
+    else:     # the first arena, p's or the whole list's, is virtual memory
+        assert count <= asked <= 2 * count + 2 * arenas and ranges <= 13 + arenas
