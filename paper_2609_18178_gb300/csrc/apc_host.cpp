@@ -41,7 +41,9 @@ apc_status fail(apc_status s, const char *fmt, ...) {
   return s;
 }
 
+// An error that is returned is not left pending with the runtime as well.
 apc_status cuda_fail(int err, const char *what) {
+  cudaGetLastError();
   return fail(APC_ECUDA, "%s: %s", what, cudaGetErrorString((cudaError_t)err));
 }
 
@@ -253,15 +255,16 @@ bool allocation_of(const void *p, uintptr_t *lo, uintptr_t *hi) {
 // a failed range query the next 1, 2, 4, ... addresses are taken one by one
 // before a range is asked for again, so that a table in virtual memory costs at
 // most log2 of its length more than its addresses (5,500 of them in PyTorch's
-// expandable segments: 850 us a commit, 1,450 with a range query for each).  Nothing is kept from one call to the next.  Returns APC_ECUDA
-// if the runtime cannot answer (for example, no device) and APC_EINVAL naming
-// the first foreign pointer (lowest address first).
+// expandable segments: 850 us a commit, 1,450 with a range query for each).
+// Nothing is kept from one call to the next.  Returns APC_ECUDA if the runtime
+// cannot answer (for example, no device) and APC_EINVAL naming the first
+// foreign pointer (lowest address first).
 apc_status check_device_pointers(const Ordered &ranges, size_t count, const char *out_name) {
   constexpr size_t kFew = 8;  // fewer pointers than this are queried one by one
   int dev = 0;
   int e = (int)cudaGetDevice(&dev);
   if (e) return cuda_fail(e, "cudaGetDevice");
-  uintptr_t lo = 0, hi = 0;     // the allocation last queried
+  uintptr_t lo = 0, hi = 0;         // the allocation last queried
   size_t one_by_one = 0, next = 1;  // addresses until a range is asked for again, and after the next failure
   apc_status st = APC_OK;
   ranges.each([&](const Range &o) {
@@ -270,7 +273,6 @@ apc_status check_device_pointers(const Ordered &ranges, size_t count, const char
     cudaPointerAttributes a;
     e = (int)cudaPointerGetAttributes(&a, p);
     if (e) {
-      cudaGetLastError();  // clear the runtime's error state of the failed query
       st = cuda_fail(e, "cudaPointerGetAttributes");
       return false;
     }

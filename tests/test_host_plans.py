@@ -98,3 +98,13 @@ def test_pointer_queries_by_kind_of_memory(lib, what, count, addresses, arenas, 
         assert asked == addresses and ranges <= 13
     else:     # the first arena, p's or the whole list's, is virtual memory
         assert count <= asked <= 2 * count + 2 * arenas and ranges <= 13 + arenas
+
+
+@pytest.mark.parametrize("what", ["commit", "digest", "count"])
+def test_a_refused_launch_leaves_no_error_pending(lib, what):
+    """An error that a call has returned is not left with the runtime for the
+    caller's next check, or this library's next launch, to find."""
+    lib.stub_reset(0, 9)
+    assert call(lib, what, 3) == 4                      # APC_ECUDA
+    assert b"launch" in lib.apc_last_error()
+    assert lib.stub_pending() == 0
