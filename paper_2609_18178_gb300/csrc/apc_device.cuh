@@ -108,15 +108,15 @@ __device__ __forceinline__ float rcp_approx(float x) {
 //             q = a*y, a/den = q + (a - q*den) * y
 // with the signs arranged so that no operand needs a negation and a zero m'
 // keeps its sign.  On this GPU both are the rounded results without exception:
-// compared with the general ones for all 1.39e9 values of x in [2^-86, 2^80),
-// for the reciprocal of all values in [2^-60, 2^10), and for the quotient of
+// compared with the general ones for all 1.77e9 values of x in [2^-86, 2^125),
+// for the reciprocal of all values in [2^-70, 2^31), and for the quotient of
 // all 2^46 pairs of significands; other exponents only scale those, since
 // nothing in the ranges below overflows or becomes subnormal.  The factors
 // 2^64 keep it so down to subnormal v' and m'; the power-of-two scaled
 // constants 1/sqrt(1-b2^t) * 2^-32 and lr/(1-b1^t) * 2^-64 take them out again.
 //
-// The form holds if |m'| + den <= 128 (the host sets limit to 128 where eps,
-// 1/sqrt(1-b2^t) and lr/(1-b1^t) are in range, see commit_scalars) and if the
+// The form holds if |m'| + den <= limit (up to 2^30, and negative where eps,
+// 1/sqrt(1-b2^t) or lr/(1-b1^t) are out of range: commit_scalars) and if the
 // quotient is not subnormal before its scaling back: |a/den| >= 2^-62, or the
 // decayed parameter is at least 2^-62, against which such a quotient vanishes.
 // One test over the group decides, by its sum of |m'| + den and its least

@@ -340,10 +340,16 @@ uint32_t commit_launch_tile(const apc::CommitEntry *e, size_t count, uint64_t fu
 }
 
 // The scalars of a launch, and the constants of adamw_group with the bounds
-// that its form needs of them: den >= eps >= 2^-50 keeps a / den below 2^121;
-// 1/sqrt(bc2) <= 2^16 keeps the root of its 2^-126 addend out of den; a
-// nonzero step in [2^-60, 2^20] keeps step * 2^-64 normal and a subnormal
-// quotient's term below 2^-106.
+// that its form needs of them.  The root of its 2^-126 addend, which enters den
+// as 1/sqrt(bc2) * 2^-95, stays under half an ulp of eps where
+// eps >= 1/sqrt(bc2) * 2^-69.  With |m'| + den <= limit = min(2^30, eps * 2^62),
+// x is below 2^125, den in [2^-69, 2^30], and a / den <= limit * 2^64 / eps at
+// most 2^126.  A nonzero step in [2^-60, 2^20] keeps step * 2^-64 normal and a
+// subnormal quotient's term below 2^-106.  Elements beyond take the general
+// operations on top of the grouped ones, so the bounds leave out only what no
+// job holds: with a fixed limit of 128 and eps >= 2^-50, 30 M elements of fp32
+// state took 162 us instead of 138 where gradients are summed instead of
+// averaged, or with eps = 1e-16, and of bf16 state 132 instead of 110.
 template <int MAXE>
 void commit_scalars(const float h[8], apc::CommitPlan<MAXE> *plan) {
   std::memcpy(plan->h, h, sizeof plan->h);
@@ -354,9 +360,8 @@ void commit_scalars(const float h[8], apc::CommitPlan<MAXE> *plan) {
     std::memcpy(&bits, &pairs[k], sizeof bits);
     plan->pair[k] = (uint64_t)bits << 32 | bits;
   }
-  const bool fits = h[4] >= 0x1p-50f && h[7] >= 1.0f && h[7] <= 0x1p16f &&
-                    (h[6] == 0.0f || (h[6] >= 0x1p-60f && h[6] <= 0x1p20f));
-  plan->limit = fits ? 128.0f : -1.0f;
+  const bool fits = h[7] >= 1.0f && h[4] >= h[7] * 0x1p-69f && (h[6] == 0.0f || (h[6] >= 0x1p-60f && h[6] <= 0x1p20f));
+  plan->limit = fits ? std::min(0x1p30f, h[4] * 0x1p62f) : -1.0f;
 }
 
 // Entries arrive without tile_begin; each batch places their tiles.

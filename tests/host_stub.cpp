@@ -22,6 +22,7 @@ struct Launch {
   int64_t count, grid, more, chained;
 };
 std::vector<Launch> g_launches;
+float g_limit;                           // the last commit plan's
 
 cudaError_t launched() {
   g_pending = g_refuse ? g_refuse : g_pending;
@@ -63,6 +64,7 @@ __attribute__((visibility("default"))) void stub_reset(uint64_t ordinary_from, i
 }
 __attribute__((visibility("default"))) long stub_runtime_queries() { return g_runtime_queries; }
 __attribute__((visibility("default"))) long stub_range_queries() { return g_range_queries; }
+__attribute__((visibility("default"))) float stub_limit() { return g_limit; }
 __attribute__((visibility("default"))) int stub_pending() { return (int)g_pending; }
 __attribute__((visibility("default"))) long stub_launches(int64_t *out, long cap) {
   for (long i = 0; i < (long)g_launches.size() && i < cap; ++i) {
@@ -106,6 +108,7 @@ namespace apc {
 
 template <int MAXE>
 int launch_commit(const CommitPlan<MAXE> &plan, int, bool, unsigned grid, void *, unsigned long long *out) {
+  g_limit = plan.limit;
   return record(plan, grid, out);
 }
 template int launch_commit(const CommitPlan<kCommitSmall> &, int, bool, unsigned, void *, unsigned long long *);

@@ -422,3 +422,13 @@ def test_masked_state_costs_no_more_than_another(layout):
             took.append(a.elapsed_time(z))
         times.append(sorted(took)[4])
     assert max(times[1:]) < 1.15 * times[0], times
+
+
+@pytest.mark.parametrize("layout", ["f32", "bf16"])
+@pytest.mark.parametrize("hp,step", [
+    (dict(eps=1e-16), 3), (dict(eps=2.0**-60), 100), (dict(eps=2.0**-66), 7), (dict(eps=2.0**-68, beta2=0.5), 100),
+    (dict(beta2=1 - 1e-12), 1), (dict(eps=1e-16, beta2=1 - 1e-9), 2), (dict(eps=2.0**20), 4), (dict(lr=1e5), 5)])
+def test_update_at_the_bounds_of_the_grouped_form(layout, hp, step):
+    """The grouped square root and quotient near the ends of the settings for
+    which the host lets them run, over states of every magnitude."""
+    test_update_over_all_magnitudes(layout, hp, step)

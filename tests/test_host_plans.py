@@ -29,22 +29,23 @@ def lib(tmp_path_factory):
     out.apc_last_error.restype = ctypes.c_char_p
     for f in (out.stub_runtime_queries, out.stub_range_queries, out.stub_launches):
         f.restype = ctypes.c_long
+    out.stub_limit.restype = ctypes.c_float
     out.stub_reset.argtypes = [ctypes.c_uint64, ctypes.c_int]
     yield out
     out.apc_set_reserved_sms(0)
 
 
-def call(lib, what, count, n=300):
+def call(lib, what, count, n=300, step=3, **hp):
     """One call over `count` tensors or buffers of n elements each; its status."""
     out = ctypes.c_void_p(BASE + (7 << 30))
     if what == "commit":
-        h = oracle.DEFAULT_HP
+        h = dict(oracle.DEFAULT_HP, **hp)
         hp = apc._HParams(h["lr"], h["beta1"], h["beta2"], h["eps"], h["weight_decay"])
         arr = (apc._Tensor * count)()
         for k in range(count):
             at = [BASE + (i << 30) + (4 if i < 3 else 2) * k * (n + 4) for i in range(5)]
             arr[k] = apc._Tensor(*at, n, k * n)
-        return lib.apc_commit_step(arr, count, ctypes.byref(hp), ctypes.c_int64(3), None, out)
+        return lib.apc_commit_step(arr, count, ctypes.byref(hp), ctypes.c_int64(step), None, out)
     arr = (apc._Buffer * count)()
     for k in range(count):
         arr[k] = apc._Buffer(BASE + 4 * k * (n + 4), n, k * n, apc.F32, 0)
@@ -108,3 +109,19 @@ def test_a_refused_launch_leaves_no_error_pending(lib, what):
     assert call(lib, what, 3) == 4                      # APC_ECUDA
     assert b"launch" in lib.apc_last_error()
     assert lib.stub_pending() == 0
+
+
+@pytest.mark.parametrize("hp,step,limit", [
+    (dict(), 1, 2.0**30), (dict(eps=1e-6, beta2=0.999), 5, 2.0**30), (dict(eps=2.0**-32), 9, 2.0**30),
+    (dict(eps=1e-15), 3, 1e-15 * 2**62), (dict(eps=1e-16), 3, 1e-16 * 2**62), (dict(eps=2.0**-60), 100, 4.0),
+    (dict(lr=0.0), 1, 2.0**30), (dict(beta2=1 - 1e-12), 1, 2.0**30), (dict(eps=300.0), 1, 2.0**30),
+    # the root of the addend in den, a step or a quotient out of binary32's normal range: the general operations
+    (dict(eps=2.0**-69, beta2=0.95), 1, -1), (dict(eps=1e-30), 5, -1), (dict(eps=1e-16, beta2=1 - 1e-15), 1, -1),
+    (dict(lr=1e-25), 5, -1), (dict(lr=1e7), 5, -1)])
+def test_bounds_of_the_grouped_update(lib, hp, step, limit):
+    """Up to which |m'| + den a group's square root and quotient keep to the
+    grouped form: what a job sets, and moments of unscaled or summed gradients,
+    lie well inside."""
+    lib.stub_reset(0, 0)
+    assert call(lib, "commit", 3, step=step, **hp) == 0
+    assert lib.stub_limit() == pytest.approx(limit, rel=1e-6)
