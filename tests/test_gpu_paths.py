@@ -432,3 +432,31 @@ def test_update_at_the_bounds_of_the_grouped_form(layout, hp, step):
     """The grouped square root and quotient near the ends of the settings for
     which the host lets them run, over states of every magnitude."""
     test_update_over_all_magnitudes(layout, hp, step)
+
+
+@pytest.mark.parametrize("scale", [0, 24, -34])
+def test_root_and_quotient_of_every_significand(scale):
+    """p = 0, g = 0 and a step of 1 leave p' = -(m' / sqrt(v')): every
+    significand of v' at an even and an odd exponent, and with them every
+    significand of den, each against an m' of random significand, compared with
+    numpy's correctly rounded root and quotient.  The grouped form's exactness
+    rests on this GPU's approximations of 1/sqrt and 1/x; the test notices a
+    changed sequence or another GPU's."""
+    n = 1 << 24
+    v = (np.arange(n, dtype=np.uint32) + np.uint32(0x3F800000)).view(np.float32) * np.float32(4.0 ** scale)  # 4^scale * [1, 4)
+    rng = np.random.default_rng(scale + 100)
+    d = {"v": dev_words((v * 2).view(np.uint32)), "g": torch.zeros(n, dtype=torch.int16, device="cuda"),
+         "w": torch.zeros(n, dtype=torch.int16, device="cuda")}
+    hp, step = dict(lr=1.0, beta1=0.5, beta2=0.5, eps=2.0**(scale - 28), weight_decay=0.0), 200
+    h8 = oracle.resolve_hparams(hp, step)
+    assert list(h8) == [0.5, 0.5, 0.5, 0.5, 2.0**(scale - 28), 1.0, 1.0, 1.0]
+    den = np.sqrt(v) + np.float32(hp["eps"])            # eps is under half an ulp
+    assert np.array_equal(den, np.sqrt(v)) and np.unique(den).size == 1 << 23
+    for _ in range(3):
+        m = (rng.integers(0, 1 << 23, size=n, dtype=np.uint32) + np.uint32(0x3F800000)).view(np.float32)
+        m *= np.float32(2.0 ** (scale - 3))
+        p = torch.zeros(n, dtype=torch.int32, device="cuda")
+        apc.commit_step([apc.TensorEntry(p, dev_words((m * 2).view(np.uint32)), d["v"].clone(), d["g"], d["w"], 0)], step, hp)
+        got = p.cpu().numpy().view(np.uint32)
+        bad = np.nonzero(got != (-(m / den)).view(np.uint32))[0]
+        assert bad.size == 0, (bad.size, bad[:5], got[bad[:5]])
