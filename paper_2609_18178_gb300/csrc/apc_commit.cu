@@ -37,7 +37,7 @@
 //    hold the tile's gradient, and the consumers read its words, and store the
 //    copy's, at their own offsets.  Where p, m and v are at odds too, all four
 //    are copied in blocks and every word is read and stored by itself,
-//    lane-consecutive.  60 M elements in 291 odd entries take 281 us, 320
+//    lane-consecutive.  60 M elements in 291 odd entries take 275 us, 320
 //    with every word by itself, 606 with element loads straight from global
 //    memory (247 at the copy rate).  Tables without such an entry run an
 //    instantiation without this code (MIS = false).
@@ -145,7 +145,7 @@ __device__ __forceinline__ uint64_t cterm(uint32_t G, uint32_t bits, uint32_t on
 // that takes the half by a dot product.
 template <uint32_t K, int HALF, bool SHARED>
 __device__ __forceinline__ uint64_t hterm(uint32_t G, uint32_t pair, uint32_t one, uint32_t top) {
-  if constexpr (SHARED) return digest_term_half<K, HALF>(G, pair, one, top);
+  if constexpr (SHARED) return digest_term_half<K, HALF>(G, pair, top);
   else return digest_term<K>(G, HALF ? pair >> 16 : pair & 0xFFFFu, one);
 }
 

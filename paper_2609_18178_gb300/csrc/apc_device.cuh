@@ -111,9 +111,11 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // compared with the general ones for all 1.77e9 values of x in [2^-86, 2^125),
 // for the reciprocal of all values in [2^-70, 2^31), and for the quotient of
 // all 2^46 pairs of significands; other exponents only scale those, since
-// nothing in the ranges below overflows or becomes subnormal.  The factors
-// 2^64 keep it so down to subnormal v' and m'; the power-of-two scaled
-// constants 1/sqrt(1-b2^t) * 2^-32 and lr/(1-b1^t) * 2^-64 take them out again.
+// nothing in the ranges below overflows or becomes subnormal.  (The tests repeat
+// the root and the reciprocal for every significand, with 5e7 pairs for the
+// quotient.)  The factors 2^64 keep it so down to subnormal v' and m'; the
+// power-of-two scaled constants 1/sqrt(1-b2^t) * 2^-32 and lr/(1-b1^t) * 2^-64
+// take them out again.
 //
 // The form holds if |m'| + den <= limit (up to 2^30, and negative where eps,
 // 1/sqrt(1-b2^t) or lr/(1-b1^t) are out of range: commit_scalars) and if the
@@ -276,7 +278,7 @@ __device__ __forceinline__ uint64_t digest_term(uint32_t gidx, uint32_t bits, ui
 // explicit multiply-adds for it).  The keyed form below saves more
 // instructions but spills at the bf16 layout's 72 registers and was no faster.
 template <uint32_t K, int HALF>
-__device__ __forceinline__ uint64_t digest_term_half(uint32_t gidx, uint32_t pair, uint32_t one, uint32_t top) {
+__device__ __forceinline__ uint64_t digest_term_half(uint32_t gidx, uint32_t pair, uint32_t top) {
   const uint32_t lo = __dp2a_lo(pair, HALF ? 0x0100u : 0x0001u, 0x7F4A7C15u);
   const uint32_t hi = gidx + (0x9E3779B9u + K), m4 = 4 * hi + 1;
   const uint32_t l1 = lo ^ m4, h1 = hi ^ top;

@@ -224,7 +224,7 @@ __device__ __forceinline__ void walk(const DigestPlan<MAXE> &plan, uint4 *stg, u
   const uint32_t one = plan.one;
   const uint64_t lo = T32 ? 0 : plan.tiles32, hi = T32 ? plan.tiles32 : plan.total_tiles;
   // this CTA's contiguous run of the kind's tiles, walked by its warps:
-  // tile t_begin + r for r = warp, warp + 32, ... below len
+  // tile t_begin + r for r = warp, warp + kWarps, ... below len
   // (the bf16 runs are dealt out from the last CTA on, so that the longer runs
   // of both kinds fall on different CTAs)
   const uint32_t c = T32 ? blockIdx.x : gridDim.x - 1 - blockIdx.x;

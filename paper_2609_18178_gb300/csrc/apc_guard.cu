@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(kCountThreads, 1) count_kernel(const __grid_co
   // this CTA's run of tiles, walked by its warps
   const uint64_t per = plan.total_tiles / gridDim.x, rem = plan.total_tiles % gridDim.x;
   const uint64_t t_begin = blockIdx.x * per + (blockIdx.x < rem ? blockIdx.x : rem);
-  const uint32_t len = (uint32_t)(per + (blockIdx.x < rem ? 1 : 0));  // 2^32 tiles are 16 TB
+  const uint32_t len = (uint32_t)(per + (blockIdx.x < rem ? 1 : 0));  // 2^32 tiles are 13 TB
   uint32_t cur = 0, r = warp;
   int slot = -1;
   uint64_t acc = 0;

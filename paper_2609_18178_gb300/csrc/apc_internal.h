@@ -150,7 +150,8 @@ static_assert(sizeof(CommitPlan<kCommitLarge>) <= 32764, "kernel parameter limit
 //    U = 4: 453 M elements of fp32 state verify in 1,427 us and 1.81 G of bf16
 //    state in 3,675 us, against 1,455 and 3,883 us for 1024 x 2, 1,430 and
 //    3,740 for 768 x 3, 1,452 and 3,879 for 512 x 4, 1,446 and 3,888 for
-//    640 x 5.
+//    640 x 5.  (All before the terms' mixed multiplies, which brought the kept
+//    shape to 1,411 and 3,650.)
 //  * U = 4 needs several tiles for every warp to be dealt out evenly: with few
 //    of them a tile of half the length spreads the work better (1 M elements
 //    of fp32 state, 1.3 long tiles per warp: 9.9 us against 12.9).  The long
@@ -274,7 +275,8 @@ template <int MAXE>
 int launch_count(const DigestPlan<MAXE> &plan, unsigned grid, void *stream, unsigned long long *out);
 
 // Resident CTAs per SM of each kernel (cudaOccupancyMaxActiveBlocksPerMultiprocessor),
-// the fewest over its instantiations.
+// the fewest over its instantiations; those that zero gradients have the threads
+// and shared memory of the others, which set it, and are not asked.
 int commit_blocks_per_sm(int *out);
 int digest_blocks_per_sm(int *out);
 int count_blocks_per_sm(int *out);
